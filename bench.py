@@ -623,7 +623,10 @@ def run_table2(args, base):
         kinds = profile_round(dart, e.h, build, 2, barrier)  # up to ~2300 launches per round: 2 fit the event pool
         lm_ms, lm_n = kinds.get("lmhead", (0.0, 0))
         n_launch = sum(v[1] for v in kinds.values())
-        launches += n_launch * args.steps
+        # the timed sequential search stops after the passes it needs (a
+        # conditional graph node), while the profiled one launches all that
+        # could be needed: only its six launches outside the passes are counted
+        launches += (6 if name == "seq_heap" else n_launch) * args.steps
         emitted = tree_to_counts(e.out_t)
         out[name] = {"us_per_round": ms[name] * 1e3, "vs_dartree": ms[name] / ms["dartree"],
                      "lmhead_launches_per_round": lm_n, "launches_per_round": n_launch,

@@ -144,16 +144,20 @@ struct dart_handle {
     float* ddt_z;
     uint64_t* ddt_part;    // [nseq * L][topk_S][Bp]
     int* ddt_ticket;       // [nseq * L]
-    // sequential correction with heap (slot 0 = the root, p + 1 = node p)
-    float* sh_tab;         // [nseq][B+1][d]
-    int* sh_ltok;          // [nseq][B+1][Bp]
+    // sequential correction with heap (SeqHeapArgs): M targets per sequence
+    // and pass, E corrected prefixes, lists of Bs slots
+    std::vector<int> scaps;
+    std::vector<DepthPlan> splans;  // [2]: M nodes per sequence, corrected and scored
+    int sh_M, sh_E, sh_Bs;
+    float* sh_tab;         // [nseq][E][d]
+    int *sh_ltok, *sh_lent;  // [nseq][E][Bs]
     float* sh_lz;
-    float* sh_llse;        // [nseq][B+1]
-    int *sh_next, *sh_npop, *sh_dlog_row;
-    float* sh_offer;
-    float* sh_zrow;        // [nseq][V]
-    uint64_t* sh_part;     // [nseq][topk_S][Bp]
-    int* sh_ticket;        // [nseq]
+    float* sh_llse;        // [nseq][E]
+    int* sh_state[2];
+    int *sh_sync, *sh_npop, *sh_dlog_row, *sh_row_ent;
+    float* sh_zrow;        // [nseq * M][V]
+    uint64_t* sh_part;     // [nseq * M][topk_S][Bp]
+    int* sh_ticket;        // [nseq * M]
     int last_kind;         // construction of the most recent round (RoundKind)
     // fused small-problem round (dart_config.fused_round): one cooperative
     // kernel of fused_G blocks, each scoring at most fused_R vocabulary rows
@@ -369,9 +373,11 @@ int plan_fused_round(dart_handle* h) {
     return DART_OK;
 }
 
-int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, std::vector<DepthPlan>& plans) {
+// (root: nodes per sequence before depth 1)
+int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, std::vector<DepthPlan>& plans,
+                int root = 1) {
     const bool tc = h->wdtype == DART_BF16;
-    caps.assign(c.L + 1, 1);
+    caps.assign(c.L + 1, root);
     for (int i = 1; i <= c.L; i++) caps[i] = std::min(c.W, caps[i - 1] * c.k);
     plans.resize(c.L + 1);
     const int tiles = (c.V + kTileM - 1) / kTileM;
@@ -546,9 +552,26 @@ int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, st
     return DART_OK;
 }
 
+// Sequential correction with heap: targets per pass (M per sequence) and
+// corrected prefixes kept (E).  One LM-head pass costs the same for 1 node
+// and for a whole node group: 16 with bf16 weights (measured on GB300,
+// V = 151936, d = 2560: 115.8 us for one, 116.8 us for sixteen), 4 with fp32.
+// E holds the B - 1 prefixes that must be corrected and as many looked ahead at.
+int plan_seq_heap(dart_handle* h) {
+    const dart_config& c = h->cfg;
+    h->sh_M = std::max(1, (h->wdtype == DART_BF16 ? kSeqHeapMaxTargets : 4) / c.nseq);
+    h->sh_E = h->sh_M > 1 ? 2 * c.B + h->sh_M : c.B + 1;
+    h->sh_Bs = (h->Bp + 3) / 4 * 4;
+    h->sh_S = cand_topk_slices(c.V, h->Bp, c.nseq * h->sh_M, h->num_sms);
+    dart_config sc = h->ccfg;
+    sc.L = 3;
+    sc.W = h->sh_M;
+    return build_plans(h, sc, h->scaps, h->splans, h->sh_M);
+}
+
 size_t max_part_floats(const dart_handle* h) {
     size_t m = 1;
-    for (const std::vector<DepthPlan>* ps : {&h->plans, &h->cplans})
+    for (const std::vector<DepthPlan>* ps : {&h->plans, &h->cplans, &h->splans})
         for (int dep = 1; dep + 1 < static_cast<int>(ps->size()); dep++) {
             const DepthPlan& p = (*ps)[dep];
             m = std::max(m, static_cast<size_t>(p.g1.S) * std::max(p.N, p.Nc) * h->cfg.d);
@@ -562,7 +585,7 @@ int alloc_workspace(dart_handle* h) {
     const size_t d = c.d;
     int rc = DART_OK;
     size_t max_nvn = 1, max_keys = 1;  // key lists x nodes; keys incl. one padding key per node
-    for (const std::vector<DepthPlan>* ps : {&h->plans, &h->cplans})
+    for (const std::vector<DepthPlan>* ps : {&h->plans, &h->cplans, &h->splans})
         for (int dep = 1; dep < static_cast<int>(ps->size()); dep++) {
             const DepthPlan& p = (*ps)[dep];
             max_nvn = std::max(max_nvn, static_cast<size_t>(p.nlist) * p.N);
@@ -615,7 +638,7 @@ int alloc_workspace(dart_handle* h) {
         DART_ALLOC(h->f_bar, kRoundBarWords)
         DART_ALLOC(h->f_abort, 1)
     }
-    const size_t ns = c.nseq, Bp = h->Bp, S1 = static_cast<size_t>(c.B) + 1;
+    const size_t ns = c.nseq, Bp = h->Bp;
     if (c.variants & DART_VARIANT_CHAIN_DDTREE) {
         DART_ALLOC(h->zrows, ns * c.L * c.V)
         DART_ALLOC(h->chain_lse, ns * c.L)
@@ -625,17 +648,22 @@ int alloc_workspace(dart_handle* h) {
         DART_ALLOC(h->ddt_ticket, ns * c.L)
     }
     if (c.variants & DART_VARIANT_SEQ_HEAP) {
-        DART_ALLOC(h->sh_tab, ns * S1 * d)
-        DART_ALLOC(h->sh_ltok, ns * S1 * Bp)
-        DART_ALLOC(h->sh_lz, ns * S1 * Bp)
-        DART_ALLOC(h->sh_llse, ns * S1)
-        DART_ALLOC(h->sh_next, ns * S1)
-        DART_ALLOC(h->sh_offer, ns * S1)
+        const size_t E = h->sh_E, M = h->sh_M, Bs = h->sh_Bs;
+        const size_t words = ns * seqheap_state_words(c.B, h->sh_E);
+        DART_ALLOC(h->sh_tab, ns * E * d)
+        DART_ALLOC(h->sh_ltok, ns * E * Bs)
+        DART_ALLOC(h->sh_lent, ns * E * Bs)
+        DART_ALLOC(h->sh_lz, ns * E * Bs)
+        DART_ALLOC(h->sh_llse, ns * E)
+        DART_ALLOC(h->sh_state[0], words)
+        DART_ALLOC(h->sh_state[1], words)
+        DART_ALLOC(h->sh_sync, 3)
         DART_ALLOC(h->sh_npop, ns)
-        DART_ALLOC(h->sh_dlog_row, ns)
-        DART_ALLOC(h->sh_zrow, ns * c.V)
-        DART_ALLOC(h->sh_part, ns * h->sh_S * Bp)
-        DART_ALLOC(h->sh_ticket, ns)
+        DART_ALLOC(h->sh_dlog_row, ns * M)
+        DART_ALLOC(h->sh_row_ent, ns * M)
+        DART_ALLOC(h->sh_zrow, ns * M * c.V)
+        DART_ALLOC(h->sh_part, ns * M * h->sh_S * Bp)
+        DART_ALLOC(h->sh_ticket, ns * M)
     }
     if (c.cand_k > 0) {
         size_t scr = 1;
@@ -665,7 +693,7 @@ int alloc_workspace(dart_handle* h) {
     if (cudaMemset(h->status, 0, sizeof(int)) != cudaSuccess) return DART_ERR_CUDA;
     if (cudaMemset(h->tree_count, 0, c.nseq * c.L * sizeof(int)) != cudaSuccess) return DART_ERR_CUDA;
     if (h->ddt_ticket && cudaMemset(h->ddt_ticket, 0, ns * c.L * sizeof(int)) != cudaSuccess) return DART_ERR_CUDA;
-    if (h->sh_ticket && cudaMemset(h->sh_ticket, 0, ns * sizeof(int)) != cudaSuccess) return DART_ERR_CUDA;
+    if (h->sh_ticket && cudaMemset(h->sh_ticket, 0, ns * h->sh_M * sizeof(int)) != cudaSuccess) return DART_ERR_CUDA;
     if (h->fused && (cudaMemset(h->f_bar, 0, kRoundBarWords * sizeof(unsigned)) != cudaSuccess ||
                      cudaMemset(h->f_abort, 0, sizeof(int)) != cudaSuccess ||
                      round_small_set_smem_limits() != cudaSuccess ||
@@ -686,7 +714,7 @@ int alloc_workspace(dart_handle* h) {
             return DART_ERR_CUDA;
     }
     if ((c.cand_k > 0 || c.variants) && cand_set_smem_limits() != cudaSuccess) return DART_ERR_CUDA;
-    if ((c.variants & DART_VARIANT_CHAIN_DDTREE) && heap_set_smem_limits() != cudaSuccess) return DART_ERR_CUDA;
+    if (c.variants && heap_set_smem_limits() != cudaSuccess) return DART_ERR_CUDA;
     if (h->wdtype == DART_BF16) {
         if (tc_set_smem_limits(h->smem_optin) != cudaSuccess) return DART_ERR_CUDA;
         if (seed_score_set_smem_limit(h->smem_optin) != cudaSuccess) return DART_ERR_CUDA;
@@ -1242,23 +1270,23 @@ int enqueue_chain_ddtree(dart_handle* h, const float* dlog, const float* anchor,
     return e == cudaSuccess ? DART_OK : DART_ERR_CUDA;
 }
 
-// Sequential correction with heap (Sec. 4.1, Table 2): B pops, each
-// correcting the popped prefix before the next: its state (head update of
-// one node per sequence) and its children over the vocabulary (LM-head,
-// merge for the log-sum-exp, the best Bp children best first).  The last pop
-// needs no correction, nor does any pop when L = 1.
-int enqueue_seq_heap(dart_handle* h, const float* dlog, const float* anchor, const dart_tree_out* out,
-                     cudaStream_t st) {
+// Sequential correction with heap (Sec. 4.1, Table 2): best-first pops, each
+// popped prefix corrected before the next pop: its state (head update) and
+// its children over the vocabulary (LM-head, merge for the log-sum-exp, the
+// best Bp children best first).  A pass corrects up to M prefixes per
+// sequence (csrc/dart_heap.cu); the step kernel between two passes says
+// whether another one is needed: at most B - 1 (the last pop needs none, nor
+// does any pop when L = 1), usually far fewer.
+SeqHeapArgs seq_heap_args(const dart_handle* h, const float* anchor, const dart_tree_out* out) {
     const dart_config& c = h->cfg;
-    const dart_config& cc = h->ccfg;
-    const DepthPlan& p = h->cplans[1];  // one node per sequence
-    const bool tc = h->wdtype == DART_BF16;
-    const size_t S1 = static_cast<size_t>(c.B) + 1;
     SeqHeapArgs a;
     std::memset(&a, 0, sizeof a);
     a.L = c.L;
     a.B = c.B;
     a.Bp = h->Bp;
+    a.Bs = h->sh_Bs;
+    a.M = h->sh_M;
+    a.E = h->sh_E;
     a.nseq = c.nseq;
     a.d = c.d;
     a.pos_offset = c.pos_offset;
@@ -1269,15 +1297,18 @@ int enqueue_seq_heap(dart_handle* h, const float* dlog, const float* anchor, con
     a.ltok = h->sh_ltok;
     a.lz = h->sh_lz;
     a.llse = h->sh_llse;
-    a.next = h->sh_next;
-    a.offer = h->sh_offer;
+    a.lent = h->sh_lent;
+    a.state[0] = h->sh_state[0];
+    a.state[1] = h->sh_state[1];
+    a.sync = h->sh_sync;
     a.npop = h->sh_npop;
     a.hin = h->hbuf[0];
-    a.HL = tc ? h->HL : nullptr;
+    a.HL = h->wdtype == DART_BF16 ? h->HL : nullptr;
     a.hout = h->hbuf[1];
     a.child_prow = h->child_prow;
     a.child_tok = h->child_tok;
     a.dlog_row = h->sh_dlog_row;
+    a.row_ent = h->sh_row_ent;
     a.tokens = out->tokens;
     a.parents = out->parents;
     a.depths = out->depths;
@@ -1286,53 +1317,128 @@ int enqueue_seq_heap(dart_handle* h, const float* dlog, const float* anchor, con
     a.scores = out->scores;
     a.mask = out->mask;
     a.status = h->status;
-    // scoring of one node per sequence, its best Bp children into slot `slot`
-    auto score = [&](int slot, const float* h32, const int* dlog_row, bool first) -> int {
-        LmheadArgs la = lmhead_args(h, cc, p, dlog, h32);
-        la.dlog_row = dlog_row;  // null: position 0 (the root's children)
-        la.gthr = first ? h->gthr : nullptr;
-        la.zout = h->sh_zrow;
-        la.zout_stride = c.V;
-        int pi = prof_begin(h, kLmhead, st);
-        cudaError_t e = tc ? launch_lmhead_tc(&h->tmE, &h->tmH[ng_index(p.NG)], la, p.smem, st) : launch_lmhead_f32(la, st);
-        prof_end(h, pi, st);
-        if (e != cudaSuccess) return DART_ERR_CUDA;
-        SelectArgs sa = select_args(h, cc, p, 1);
-        sa.gthr = la.gthr;
-        sa.lse_hist = h->sh_llse + slot;
-        sa.lse_hist_stride = static_cast<long long>(S1);
-        pi = prof_begin(h, kSelect, st);
-        e = launch_merge_select(sa, st);
-        prof_end(h, pi, st);
-        if (e != cudaSuccess) return DART_ERR_CUDA;
-        pi = prof_begin(h, kRowTopk, st);
-        e = launch_row_topk_by_value(h->sh_zrow, c.nseq, c.V, h->Bp, h->sh_S, h->sh_ltok + slot * h->Bp,
-                                     h->sh_lz + slot * h->Bp, static_cast<long long>(S1) * h->Bp, h->sh_part,
-                                     h->sh_ticket, st);
-        prof_end(h, pi, st);
-        return e == cudaSuccess ? DART_OK : DART_ERR_CUDA;
-    };
-    int pi = prof_begin(h, kPrep, st);
-    cudaError_t e = launch_prep_anchor(anchor, c.nseq, c.d, h->hbuf[0], tc ? h->HL : nullptr, kNPadMax, h->gthr,
-                                       kNPadMax, st);
+    return a;
+}
+
+// Scoring of the pass's targets, the best Bp children of each into its entry.
+int enqueue_seq_score(dart_handle* h, const float* dlog, const float* h32, cudaStream_t st) {
+    const dart_config& cc = h->ccfg;
+    const DepthPlan& p = h->splans[2];
+    LmheadArgs la = lmhead_args(h, cc, p, dlog, h32);
+    // every row is a "sequence" of one node with its own drafter row
+    la.P = 1;
+    la.dlog_seq_stride = 0;
+    la.dlog_row = h->sh_dlog_row;
+    la.zout = h->sh_zrow;
+    la.zout_stride = cc.V;
+    int pi = prof_begin(h, kLmhead, st);
+    cudaError_t e = h->wdtype == DART_BF16 ? launch_lmhead_tc(&h->tmE, &h->tmH[ng_index(p.NG)], la, p.smem, st)
+                                           : launch_lmhead_f32(la, st);
     prof_end(h, pi, st);
     if (e != cudaSuccess) return DART_ERR_CUDA;
-    int rc = score(0, h->hbuf[0], nullptr, true);
-    if (rc != DART_OK) return rc;
-    for (int t = 0; t < c.B; t++) {
-        pi = prof_begin(h, kSeqStep, st);
-        e = launch_seqheap_step(a, t, st);
-        prof_end(h, pi, st);
-        if (e != cudaSuccess) return DART_ERR_CUDA;
-        if (c.L == 1 || t + 1 == c.B) continue;
-        rc = enqueue_head_update(h, cc, p, h->hbuf[0], h->hbuf[1], false, st);
-        if (rc == DART_OK) rc = score(t + 1, h->hbuf[1], h->sh_dlog_row, false);
-        if (rc != DART_OK) return rc;
-    }
-    pi = prof_begin(h, kSeqEmit, st);
-    e = launch_seqheap_emit(a, st);
+    pi = prof_begin(h, kSelect, st);
+    e = launch_merge_lse(h->part_ms, p.N, p.nV, h->sh_row_ent, h->sh_llse, st);
+    prof_end(h, pi, st);
+    if (e != cudaSuccess) return DART_ERR_CUDA;
+    pi = prof_begin(h, kRowTopk, st);
+    e = launch_row_topk_by_value(h->sh_zrow, p.N, cc.V, h->Bp, h->sh_S, h->sh_ltok, h->sh_lz, h->sh_Bs, h->sh_part,
+                                 h->sh_ticket, st, h->sh_row_ent);
     prof_end(h, pi, st);
     return e == cudaSuccess ? DART_OK : DART_ERR_CUDA;
+}
+
+int enqueue_seq_step(dart_handle* h, const SeqHeapArgs& a, cudaGraphConditionalHandle cond, bool has_cond,
+                     cudaStream_t st) {
+    const int pi = prof_begin(h, kSeqStep, st);
+    const cudaError_t e = launch_seqheap_step(a, cond, has_cond, st);
+    prof_end(h, pi, st);
+    return e == cudaSuccess ? DART_OK : DART_ERR_CUDA;
+}
+
+// Up to the first search step: the root's children.
+int enqueue_seq_begin(dart_handle* h, const float* dlog, const SeqHeapArgs& a, cudaGraphConditionalHandle cond,
+                      bool has_cond, cudaStream_t st) {
+    const int pi = prof_begin(h, kPrep, st);
+    const cudaError_t e = launch_seqheap_init(a, st);
+    prof_end(h, pi, st);
+    if (e != cudaSuccess) return DART_ERR_CUDA;
+    int rc = enqueue_seq_score(h, dlog, h->hbuf[0], st);
+    if (rc == DART_OK) rc = enqueue_seq_step(h, a, cond, has_cond, st);
+    return rc;
+}
+
+// One pass and the search step after it.
+int enqueue_seq_pass(dart_handle* h, const float* dlog, const SeqHeapArgs& a, cudaGraphConditionalHandle cond,
+                     bool has_cond, cudaStream_t st) {
+    int rc = enqueue_head_update(h, h->ccfg, h->splans[2], h->hbuf[0], h->hbuf[1], false, st);
+    if (rc == DART_OK) rc = enqueue_seq_score(h, dlog, h->hbuf[1], st);
+    if (rc == DART_OK) rc = enqueue_seq_step(h, a, cond, has_cond, st);
+    return rc;
+}
+
+int enqueue_seq_emit(dart_handle* h, const SeqHeapArgs& a, cudaStream_t st) {
+    const int pi = prof_begin(h, kSeqEmit, st);
+    const cudaError_t e = launch_seqheap_emit(a, st);
+    prof_end(h, pi, st);
+    return e == cudaSuccess ? DART_OK : DART_ERR_CUDA;
+}
+
+// The search as a fixed sequence of launches (while profiling or when the
+// caller captures the stream): as many passes as can be needed.
+int enqueue_seq_heap(dart_handle* h, const float* dlog, const float* anchor, const dart_tree_out* out,
+                     cudaStream_t st) {
+    const SeqHeapArgs a = seq_heap_args(h, anchor, out);
+    const int passes = h->cfg.L > 1 ? h->cfg.B - 1 : 0;
+    int rc = enqueue_seq_begin(h, dlog, a, cudaGraphConditionalHandle(), false, st);
+    for (int t = 0; t < passes && rc == DART_OK; t++)
+        rc = enqueue_seq_pass(h, dlog, a, cudaGraphConditionalHandle(), false, st);
+    return rc == DART_OK ? enqueue_seq_emit(h, a, st) : rc;
+}
+
+// The search as a graph whose passes are the body of a conditional (while)
+// node, so that only the passes that are needed run.
+int capture_seq_heap(dart_handle* h, const float* dlog, const float* anchor, const dart_tree_out* out,
+                     cudaGraph_t* graph) {
+    *graph = nullptr;
+    const SeqHeapArgs a = seq_heap_args(h, anchor, out);
+    cudaStream_t cs = h->cap_stream;
+    cudaGraph_t g = nullptr, got = nullptr;
+    cudaGraphConditionalHandle cond;
+    if (cudaGraphCreate(&g, 0) != cudaSuccess) return DART_ERR_CUDA;
+    *graph = g;
+    if (cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault) != cudaSuccess ||
+        cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+        return DART_ERR_CUDA;
+    int rc = enqueue_seq_begin(h, dlog, a, cond, true, cs);
+    std::vector<cudaGraphNode_t> ends;
+    if (rc == DART_OK) {
+        cudaStreamCaptureStatus status;
+        const cudaGraphNode_t* deps = nullptr;
+        size_t nd = 0;
+        if (cudaStreamGetCaptureInfo(cs, &status, nullptr, nullptr, &deps, nullptr, &nd) != cudaSuccess)
+            rc = DART_ERR_CUDA;
+        else
+            ends.assign(deps, deps + nd);
+    }
+    if (cudaStreamEndCapture(cs, &got) != cudaSuccess && rc == DART_OK) rc = DART_ERR_CUDA;
+    if (rc != DART_OK) return rc;
+    cudaGraphNodeParams np = {cudaGraphNodeTypeConditional};
+    np.conditional.handle = cond;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    cudaGraphNode_t loop;
+    if (cudaGraphAddNode(&loop, g, ends.data(), nullptr, ends.size(), &np) != cudaSuccess) return DART_ERR_CUDA;
+    if (cudaStreamBeginCaptureToGraph(cs, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+        return DART_ERR_CUDA;
+    rc = enqueue_seq_pass(h, dlog, a, cond, true, cs);
+    if (cudaStreamEndCapture(cs, &got) != cudaSuccess && rc == DART_OK) rc = DART_ERR_CUDA;
+    if (rc != DART_OK) return rc;
+    if (cudaStreamBeginCaptureToGraph(cs, g, &loop, nullptr, 1, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+        return DART_ERR_CUDA;
+    rc = enqueue_seq_emit(h, a, cs);
+    if (cudaStreamEndCapture(cs, &got) != cudaSuccess && rc == DART_OK) rc = DART_ERR_CUDA;
+    return rc;
 }
 
 int check_inputs(const dart_handle* h, const float* dlog, const float* anchor, bool need_anchor) {
@@ -1409,9 +1515,14 @@ int run_round(dart_handle* h, int kind, const float* dlog, const float* anchor, 
         }
     }
     cudaGraph_t graph = nullptr;
-    if (cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return DART_ERR_CUDA;
-    rc = enqueue_kind(h, kind, dlog, anchor, out, h->cap_stream);
-    cudaError_t ce = cudaStreamEndCapture(h->cap_stream, &graph);
+    cudaError_t ce = cudaSuccess;
+    if (kind == kRoundSeqHeap && h->cfg.L > 1 && h->cfg.B > 1) {
+        rc = capture_seq_heap(h, dlog, anchor, out, &graph);
+    } else {
+        if (cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return DART_ERR_CUDA;
+        rc = enqueue_kind(h, kind, dlog, anchor, out, h->cap_stream);
+        ce = cudaStreamEndCapture(h->cap_stream, &graph);
+    }
     if (rc != DART_OK || ce != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
         finish_round(h, kind, false);
@@ -1509,8 +1620,8 @@ int dart_init_head(dart_handle** out, const dart_config* cfg, int wdtype, const 
         h->ccfg.k = 1;
         h->Bp = std::min(cfg->B, cfg->V);
         h->ddt_S = cand_topk_slices(cfg->V, h->Bp, cfg->nseq * cfg->L, sms);
-        h->sh_S = cand_topk_slices(cfg->V, h->Bp, cfg->nseq, sms);
         if (rc == DART_OK) rc = build_plans(h, h->ccfg, h->ccaps, h->cplans);
+        if (rc == DART_OK && (cfg->variants & DART_VARIANT_SEQ_HEAP)) rc = plan_seq_heap(h);
         if (rc == DART_OK && (cfg->variants & DART_VARIANT_CHAIN_DDTREE) &&
             ddtree_smem(cfg->L, h->Bp, cfg->B) > optin)
             rc = DART_ERR_UNSUPPORTED;

@@ -122,7 +122,7 @@ __device__ __forceinline__ void for_row(const float* x, int V, F&& f) {
 // waits) selects the K largest of the S K published keys.
 __global__ void __launch_bounds__(kTopkThreads)
     cand_topk_kernel(const float* dlog, int V, int K, int S, int* cand_tok, uint64_t* part, int* ticket,
-                     int by_value, long long out_stride, float* out_val) {
+                     int by_value, long long out_stride, float* out_val, const int* out_row) {
     pdl_trigger();
     pdl_wait();
     extern __shared__ uint64_t csm[];
@@ -137,6 +137,8 @@ __global__ void __launch_bounds__(kTopkThreads)
     __shared__ int cnt[2];  // [0] keys taken into out, [1] keys gathered into coll
     __shared__ int last;
     const int row = blockIdx.x / S, sl = blockIdx.x % S;
+    const int orow = out_row ? __ldcg(out_row + row) : row;
+    if (orow < 0) return;  // nothing to select for this row
     const int v0 = static_cast<int>(static_cast<long long>(V) * sl / S);
     const int Vs = static_cast<int>(static_cast<long long>(V) * (sl + 1) / S) - v0;
     const int Kl = min(K, Vs);  // keys this block selects from its slice
@@ -277,8 +279,8 @@ __global__ void __launch_bounds__(kTopkThreads)
         } else {
             for (int j = 0; j < K; j++) r += key_idx(out[j]) < tk;
         }
-        cand_tok[static_cast<size_t>(row) * out_stride + r] = static_cast<int>(tk);
-        if (out_val) out_val[static_cast<size_t>(row) * out_stride + r] = key_val(out[i]);
+        cand_tok[static_cast<size_t>(orow) * out_stride + r] = static_cast<int>(tk);
+        if (out_val) out_val[static_cast<size_t>(orow) * out_stride + r] = key_val(out[i]);
     }
 }
 
@@ -435,13 +437,15 @@ cudaError_t cand_set_smem_limits() {
 cudaError_t launch_cand_topk(const float* dlog, int rows, int V, int K, int S, int* cand_tok, uint64_t* part,
                              int* ticket, cudaStream_t st) {
     return launch_pdl(cand_topk_kernel, dim3(rows * S), dim3(kTopkThreads), cand_topk_smem(K), st, dlog, V, K, S,
-                      cand_tok, part, ticket, 0, static_cast<long long>(K), static_cast<float*>(nullptr));
+                      cand_tok, part, ticket, 0, static_cast<long long>(K), static_cast<float*>(nullptr),
+                      static_cast<const int*>(nullptr));
 }
 
 cudaError_t launch_row_topk_by_value(const float* x, int rows, int V, int K, int S, int* tok, float* val,
-                                     long long out_stride, uint64_t* part, int* ticket, cudaStream_t st) {
+                                     long long out_stride, uint64_t* part, int* ticket, cudaStream_t st,
+                                     const int* out_row) {
     return launch_pdl(cand_topk_kernel, dim3(rows * S), dim3(kTopkThreads), cand_topk_smem(K), st, x, V, K, S, tok,
-                      part, ticket, 1, out_stride, val);
+                      part, ticket, 1, out_stride, val, out_row);
 }
 
 cudaError_t launch_cand_score(const CandArgs& a, cudaStream_t st) {

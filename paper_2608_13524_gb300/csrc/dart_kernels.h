@@ -97,7 +97,7 @@ struct LmheadArgs {
     int e_tiled;          // the E tensor map is over the tiled copy (launch_retile), not [V][d]
     int DS;               // fp32 kernel: blocks (one cluster) sharing a vocabulary range, each a slice of d
     // optional (null: unused)
-    const int* dlog_row;  // [nseq] drafter row of each sequence's nodes (replaces dlog_row_off / V)
+    const int* dlog_row;  // [N / P] drafter row of each sequence's nodes (replaces dlog_row_off / V)
     float* zout;          // z[n][v] written to zout[n * zout_stride + v] (node groups <= 64)
     long long zout_stride;
     const float* seed_y;  // [N][seed_R] seed scores (launch_seed_score): the filter starts from each
@@ -216,6 +216,8 @@ struct SelectArgs {
     long long lse_hist_stride;
 };
 cudaError_t launch_merge_select(const SelectArgs& a, cudaStream_t st);
+// log-sum-exp of node n's nV partials to lse[row_ent[n]], where row_ent[n] >= 0
+cudaError_t launch_merge_lse(const float2* part_ms, int N, int nV, const int* row_ent, float* lse, cudaStream_t st);
 int merge_select_smem(int nV, int klist, int k, int W);
 cudaError_t select_set_smem_limits();  // the device maximum (set_max_dynamic_smem)
 
@@ -241,9 +243,11 @@ struct CandArgs {
 cudaError_t launch_cand_topk(const float* dlog, int rows, int V, int K, int S, int* cand_tok, uint64_t* part,
                              int* ticket, cudaStream_t st);
 // The same selection over rows of any fp32 values x [rows][V], written best
-// first (value desc, index asc): tok / val [rows][out_stride], K per row.
+// first (value desc, index asc): tok / val [rows][out_stride], K per row;
+// with out_row, row r's to row out_row[r] of tok / val (< 0: not selected).
 cudaError_t launch_row_topk_by_value(const float* x, int rows, int V, int K, int S, int* tok, float* val,
-                                     long long out_stride, uint64_t* part, int* ticket, cudaStream_t st);
+                                     long long out_stride, uint64_t* part, int* ticket, cudaStream_t st,
+                                     const int* out_row = nullptr);
 int cand_topk_slices(int V, int K, int rows, int num_sms);
 cudaError_t launch_cand_score(const CandArgs& a, cudaStream_t st);
 int cand_topk_smem(int K);
@@ -281,34 +285,43 @@ struct DdtArgs {
 int ddtree_smem(int L, int Bp, int B);
 cudaError_t heap_set_smem_limits();    // the device maximum
 cudaError_t launch_ddtree(const DdtArgs& a, cudaStream_t st);
-// Sequential correction with heap: per sequence, slot 0 = the root and slot
-// p + 1 = popped node p: state tab [nseq][B+1][d], sorted children ltok / lz
-// [nseq][B+1][Bp] (value order) with their log-sum-exp llse [nseq][B+1],
-// cursor next and offer [nseq][B+1], pops npop [nseq]; the output rows are
-// written in pop order.  hin / HL (rows s, bhalf + s): the head's input for
-// the popped prefix; hout: the head's output; child_prow / child_tok /
-// dlog_row [nseq]: the head update's and the LM-head's per-sequence inputs.
+// Sequential correction with heap (dart_heap.cu): M targets per sequence and
+// pass, at most E corrected prefixes (entries; entry 0 the root) per
+// sequence: states tab [nseq][E][d], sorted children ltok / lz [nseq][E][Bs]
+// (value order, the first Bp of Bs) with their log-sum-exp llse [nseq][E],
+// lent [nseq][E][Bs] the entry of an entry's child; state: two buffers of
+// [nseq][seqheap_state_words] words; sync: 3 words; pops npop [nseq]; the output rows are
+// written in pop order.  Row s * M + m is target m of sequence s: hin / HL (rows r,
+// bhalf + r) the head's input, hout its output; child_prow / child_tok /
+// dlog_row / row_ent [nseq * M] the head update's, the LM-head's and the
+// lists' indices (row_ent -1: no target).
+constexpr int kSeqHeapMaxTargets = 16;
 struct SeqHeapArgs {
-    int L, B, Bp, nseq, d, pos_offset, bhalf;
+    int L, B, Bp, Bs, M, E, nseq, d, pos_offset, bhalf;
     float beta;
-    const float* anchor;  // [nseq][d] r_0 (slot 0 of the table)
+    const float* anchor;  // [nseq][d] r_0
     float* tab;
     const int* ltok;
     const float* lz;
     const float* llse;
-    int* next;
-    float* offer;
+    int* lent;
+    int* state[2];
+    int* sync;
     int* npop;
     float* hin;
     __nv_bfloat16* HL;
     const float* hout;
-    int *child_prow, *child_tok, *dlog_row;
+    int *child_prow, *child_tok, *dlog_row, *row_ent;
     int *tokens, *parents, *depths, *pos_ids, *n_nodes;
     float* scores;
     uint64_t* mask;
     int* status;
 };
-cudaError_t launch_seqheap_step(const SeqHeapArgs& a, int t, cudaStream_t st);
+int seqheap_step_smem(int B, int E);
+int seqheap_state_words(int B, int E);
+cudaError_t launch_seqheap_init(const SeqHeapArgs& a, cudaStream_t st);
+// has_cond: sets the graph conditional to whether another pass is needed
+cudaError_t launch_seqheap_step(const SeqHeapArgs& a, cudaGraphConditionalHandle cond, bool has_cond, cudaStream_t st);
 cudaError_t launch_seqheap_emit(const SeqHeapArgs& a, cudaStream_t st);
 
 // The whole round of a small fp32 problem in one cooperative kernel

@@ -129,6 +129,30 @@ __global__ void __launch_bounds__(kSelThreads) merge_select_kernel(const SelectA
     select_frontier(a, s, prev_count, keys, ctok, surv, top, &thr, hist, scal, redi);
 }
 
+// Only the log-sum-exp of each node (the same arithmetic), of the nodes with
+// row_ent[n] >= 0, to lse[row_ent[n]] (sequential search).
+__global__ void __launch_bounds__(kSelThreads) merge_lse_kernel(const float2* part_ms, int nV, const int* row_ent,
+                                                                float* lse) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ float redf[32];
+    __shared__ float redm[32];
+    const int n = blockIdx.x, tid = threadIdx.x;
+    const int ent = __ldcg(row_ent + n);
+    if (ent < 0) return;
+    const float2* ms = part_ms + static_cast<size_t>(n) * nV;
+    float2 acc = make_float2(-INFINITY, 0.0f);
+    for (int r = tid + 2 * kSelThreads; r < nV; r += kSelThreads) acc = lse_merge(acc, __ldcg(ms + r));
+    for (int r = tid; r < min(nV, 2 * kSelThreads); r += kSelThreads) acc = lse_merge(acc, __ldcg(ms + r));
+    const float m = warp_max(acc.x);
+    if ((tid & 31) == 0) redm[tid >> 5] = m;
+    __syncthreads();
+    float gm = -INFINITY;
+    for (int i = 0; i < kSelThreads / 32; i++) gm = fmaxf(gm, redm[i]);
+    const float ssum = block_sum_float(acc.x == -INFINITY ? 0.0f : acc.y * __expf(acc.x - gm), redf);
+    if (tid == 0) lse[ent] = gm == -INFINITY ? -INFINITY : gm + logf(ssum);
+}
+
 __global__ void __launch_bounds__(kEmitThreads) prune_emit_kernel(const EmitArgs a) {
     pdl_trigger();
     pdl_wait();
@@ -323,6 +347,10 @@ cudaError_t select_set_smem_limits() { return set_max_dynamic_smem(reinterpret_c
 cudaError_t launch_merge_select(const SelectArgs& a, cudaStream_t st) {
     const int smem = merge_select_smem(a.nV, a.klist, a.k, a.W);
     return launch_pdl(merge_select_kernel, dim3(a.N), dim3(kSelThreads), smem, st, a);
+}
+
+cudaError_t launch_merge_lse(const float2* part_ms, int N, int nV, const int* row_ent, float* lse, cudaStream_t st) {
+    return launch_pdl(merge_lse_kernel, dim3(N), dim3(kSelThreads), 0, st, part_ms, nV, row_ent, lse);
 }
 
 cudaError_t launch_prune_emit(const EmitArgs& a, cudaStream_t st) {

@@ -181,3 +181,37 @@ def test_full_size_best_first_parity(dart, cfg):
     ref2 = oracle.seq_heap(cfg, x["Wi"], x["Wo"], x["E"], x["Dlog"], x["h0"])
     rep2 = compare_pop_order_tree(cfg, ref2, g2, tol, corrected_path_score(cfg, x))
     print(cfg.name, "seq heap", rep2)
+
+
+# targets per pass (16 / nseq with bf16 weights, 4 / nseq with fp32) and the
+# sizes at which a pass or a list is cut: (nseq, V, L, B, wdtype)
+PASSES = [(3, 900, 5, 33, "bf16"), (1, 70, 2, 2, "bf16"), (16, 300, 3, 18, "bf16"), (17, 300, 3, 9, "bf16"),
+          (2, 800, 4, 31, "f32"), (1, 5000, 9, 130, "bf16"), (1, 6, 3, 40, "bf16")]
+
+
+@pytest.mark.parametrize("nseq,V,L,B,wdtype", PASSES)
+def test_seq_heap_passes(dart, nseq, V, L, B, wdtype):
+    """The search that corrects several prefixes a pass pops what the oracle's
+    one-prefix-at-a-time search pops, as a graph (conditional passes) and as
+    the fixed launch sequence that a capturing caller gets."""
+    cfg = Config("heap-pass", nseq, V, 128, L, 2, 2, B, wdtype, 0.8, 75, variants=2)
+    x = make_inputs(cfg)
+    dx = to_device(cfg, x)
+    eng = dart.Dart(cfg, dx["Wi"], dx["Wo"], dx["E"])
+    try:
+        g = tree_to_numpy(eng.build_seq_heap(dx["Dlog"], dx["h0"]))
+        assert dart.dart_status_sync(eng.h) == 0
+        ref = oracle.seq_heap(cfg, x["Wi"], x["Wo"], x["E"], x["Dlog"], x["h0"])
+        compare_pop_order_tree(cfg, ref, g, tol_of(cfg), corrected_path_score(cfg, x))
+        cg = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(cg):
+            out = eng.build_seq_heap(dx["Dlog"], dx["h0"])
+        for t in out.values():
+            t.zero_()
+        cg.replay()
+        torch.cuda.synchronize()
+        for k, v in tree_to_numpy(out).items():
+            np.testing.assert_array_equal(v, g[k], err_msg=k)
+        assert dart.dart_status_sync(eng.h) == 0
+    finally:
+        eng.close()
