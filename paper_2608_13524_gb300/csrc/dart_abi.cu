@@ -114,7 +114,7 @@ struct dart_handle {
     int* node_tok;
     int *tree_tok, *tree_parent, *tree_count;
     float* tree_score;
-    int *child_prow, *child_tok, *seq_ticket, *status;
+    int *child_prow, *child_tok, *status;
     uint64_t* gthr;  // [L][kNPadMax] cross-CTA top-k bounds of every depth, zeroed per round
     float* bound_y;     // [kNPadMax][kBoundR] seed scores less their error bounds (topk_bound)
     int* cand_tok;   // [nseq][L][cand_k] candidate sets C_d (cand_k > 0)
@@ -616,7 +616,6 @@ int alloc_workspace(dart_handle* h) {
     DART_ALLOC(h->tree_count, static_cast<size_t>(c.nseq) * c.L)
     DART_ALLOC(h->child_prow, kNPadMax)
     DART_ALLOC(h->child_tok, kNPadMax)
-    DART_ALLOC(h->seq_ticket, c.nseq)
     DART_ALLOC(h->status, 1)
     DART_ALLOC(h->gthr, static_cast<size_t>(c.L) * kNPadMax)
     if (h->wdtype == DART_BF16) DART_ALLOC(h->bound_y, static_cast<size_t>(kNPadMax) * kBoundR)
@@ -689,7 +688,6 @@ int alloc_workspace(dart_handle* h) {
         if (cudaMemset(h->X32, 0, kNPadMax * 2 * d * 4) != cudaSuccess) return DART_ERR_CUDA;
         if (cudaMemset(h->A32, 0, kNPadMax * d * 4) != cudaSuccess) return DART_ERR_CUDA;
     }
-    if (cudaMemset(h->seq_ticket, 0, c.nseq * sizeof(int)) != cudaSuccess) return DART_ERR_CUDA;
     if (cudaMemset(h->status, 0, sizeof(int)) != cudaSuccess) return DART_ERR_CUDA;
     if (cudaMemset(h->tree_count, 0, c.nseq * c.L * sizeof(int)) != cudaSuccess) return DART_ERR_CUDA;
     if (h->ddt_ticket && cudaMemset(h->ddt_ticket, 0, ns * c.L * sizeof(int)) != cudaSuccess) return DART_ERR_CUDA;
@@ -702,7 +700,7 @@ int alloc_workspace(dart_handle* h) {
     // one-time kernel attributes
     int max_sel = 0;
     for (int dep = 1; dep <= c.L; dep++)
-        max_sel = std::max(max_sel, merge_select_smem(h->plans[dep].nlist, h->plans[dep].klist, c.k, c.W));
+        max_sel = std::max(max_sel, merge_select_smem(h->plans[dep].P, h->plans[dep].nlist, c.k));
     if (max_sel > h->smem_optin) return DART_ERR_UNSUPPORTED;
     if (select_set_smem_limits() != cudaSuccess) return DART_ERR_CUDA;
     if (c.cand_k > 0) {
@@ -883,7 +881,6 @@ SelectArgs select_args(const dart_handle* h, const dart_config& c, const DepthPl
     sa.tree_count = h->tree_count;
     sa.child_prow = h->child_prow;
     sa.child_tok = h->child_tok;
-    sa.seq_ticket = h->seq_ticket;
     sa.status = h->status;
     return sa;
 }

@@ -210,7 +210,6 @@ struct SelectArgs {
     int* tree_count;       // [nseq][L]
     int* child_prow;       // [nseq*Pn]
     int* child_tok;
-    int* seq_ticket;       // [nseq]
     int* status;
     float* lse_hist;       // optional: node n's log-sum-exp also to lse_hist[n * lse_hist_stride]
     long long lse_hist_stride;
@@ -218,7 +217,7 @@ struct SelectArgs {
 cudaError_t launch_merge_select(const SelectArgs& a, cudaStream_t st);
 // log-sum-exp of node n's nV partials to lse[row_ent[n]], where row_ent[n] >= 0
 cudaError_t launch_merge_lse(const float2* part_ms, int N, int nV, const int* row_ent, float* lse, cudaStream_t st);
-int merge_select_smem(int nV, int klist, int k, int W);
+int merge_select_smem(int P, int nV, int k);
 cudaError_t select_set_smem_limits();  // the device maximum (set_max_dynamic_smem)
 
 // candidate-restricted scoring (dart_cand.cu)

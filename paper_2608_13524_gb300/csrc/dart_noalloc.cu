@@ -166,7 +166,6 @@ extern "C" int dart_expand_root_noalloc(const dart_config* cfg, const void* E, c
     int* tree_parent = reinterpret_cast<int*>(take(size_t(N) * c.W * 4));
     int* child_prow = reinterpret_cast<int*>(take(size_t(N) * Pn * 4));
     int* child_tok = reinterpret_cast<int*>(take(size_t(N) * Pn * 4));
-    int* seq_ticket = reinterpret_cast<int*>(take(size_t(N) * 4));
     uint64_t* gthr = reinterpret_cast<uint64_t*>(take(size_t(N) * 8));
     if (off > kScratchBytes) return DART_ERR_INVALID;
 
@@ -176,9 +175,7 @@ extern "C" int dart_expand_root_noalloc(const dart_config* cfg, const void* E, c
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // the shared array keeps the previous call's contents: zero what must start at zero
-    if (cudaMemsetAsync(seq_ticket, 0, size_t(N) * 4, st) != cudaSuccess ||
-        cudaMemsetAsync(status, 0, 4, st) != cudaSuccess)
-        return DART_ERR_CUDA;
+    if (cudaMemsetAsync(status, 0, 4, st) != cudaSuccess) return DART_ERR_CUDA;
     if (launch_prep_anchor(anchor_h, N, c.d, h32, HL, kBhalfNoAlloc, gthr, N, st) != cudaSuccess) return DART_ERR_CUDA;
 
     LmheadArgs la;
@@ -229,7 +226,6 @@ extern "C" int dart_expand_root_noalloc(const dart_config* cfg, const void* E, c
     sa.tree_count = front_count;
     sa.child_prow = child_prow;
     sa.child_tok = child_tok;
-    sa.seq_ticket = seq_ticket;
     sa.status = status;
     if (launch_merge_select(sa, st) != cudaSuccess) return DART_ERR_CUDA;
     {

@@ -1,11 +1,10 @@
 // Selection, emission and small elementwise kernels of the DARTree path.
 //
 //   merge_select  (Algorithm 1, scoring + "retain the global top-W"):
-//       one block per expanded node merges the LM-head kernel's per-CTA
-//       partials into log-sum-exp and the node's top-k children,
-//       log q~ = min(z - lse, 0); the last block of each sequence (atomic
-//       ticket, no waiting) then scores the candidates with Eq. 5 and keeps
-//       the top-W as S_d.
+//       one cluster of blocks per sequence merges the LM-head kernel's
+//       per-CTA partials into every node's log-sum-exp and top-k children,
+//       log q~ = min(z - lse, 0), scores them with Eq. 5, and its block 0
+//       keeps the top-W as S_d.
 //   prune_emit    (Algorithm 1 final step + Lemma 1, Sec. 3.3 flattening):
 //       one block per sequence: global top-B by (score desc, node id asc),
 //       compaction in id order, parent remap, depths, position ids and the
@@ -13,11 +12,11 @@
 //   prep / gather / silu / gather_silu / residual_norm: the elementwise parts
 //       of the fallback correction head around the two GEMMs (gather_silu
 //       adds the per-token row of the split first layer's table).
+#include <algorithm>
 #include <cstdlib>
 
 #include "dart_device.cuh"
 #include "dart_emit.cuh"
-#include "dart_frontier.cuh"
 #include "dart_kernels.h"
 
 namespace dart {
@@ -27,106 +26,306 @@ namespace {
 constexpr int kSelThreads = 512;
 constexpr int kEmitThreads = 1024;
 
-__global__ void __launch_bounds__(kSelThreads) merge_select_kernel(const SelectArgs a) {
+// merge_select: one cluster of blocks per sequence; a block merges the
+// LM-head's partials of several nodes at once, kPer threads each (a thread
+// per vocabulary range), and the frontier's candidates are handed to block 0
+// of the cluster through distributed shared memory.  The kernel is on every
+// depth's serial chain and bound by latency: dependent round trips, barriers,
+// and the fetch of its own instructions, which are cold at every depth (the
+// LM-head between two launches is larger than the instruction caches), so the
+// code is kept small: loops are not unrolled, only the first four keys of
+// every (sorted) list are read at once and more only from lists whose fourth
+// key is still a candidate, a threshold from group maxima (k <= 16) replaces
+// ranked list heads, and up to 16 parents' candidates are ranked by binary
+// searches in their sorted lists.
+// Measured on GB300 against one block per node that read every list whole and
+// handed over through global memory and an atomic ticket (µs per round, same
+// box): 8 nodes, k = 8, d = 2560 2178 -> 2080; 16 nodes, k = 16, d = 4096
+// 3479 -> 3427; 64 nodes, k = 64 2771 -> 2714; 3 x 11 nodes 591 -> 564; 8 x 32
+// nodes and candidate sets (where the W_i GEMM beside it is longer) -0.5 %.
+constexpr int kMergeCluster = 16;     // blocks per cluster, at most
+constexpr int kMergeThreads = 1024;
+constexpr int kGroupMaxK = 16;        // threshold from group maxima up to this k
+constexpr int kMergeSearchP = 16;     // frontier by binary searches up to this many parents
+
+__device__ __forceinline__ void st_cluster_u64(uint32_t local, uint32_t rank, uint64_t v) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(remote), "l"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster_s32(uint32_t local, uint32_t rank, int v) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
+}
+
+// More than kRankMax keys reach the threshold (many equal scores): the kk
+// largest of the n keys by radix select, into surv (unsorted).
+__device__ __noinline__ void radix_survivors(const uint64_t* keys, int n, int kk, uint64_t* surv, uint32_t* hist,
+                                             int* scal) {
+    const uint64_t kth = block_kth_largest(keys, n, kk, hist, scal);
+    if (threadIdx.x == 0) scal[2] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint64_t x = keys[i];
+        if (x != 0ull && x >= kth) surv[atomicAdd(&scal[2], 1)] = x;
+    }
+    __syncthreads();
+}
+
+// Keys above x among l[0..m) (16-byte aligned; l[m] = 0 when m is odd).
+__device__ __forceinline__ int count_above(const uint64_t* l, int m, uint64_t x) {
+    const ulonglong2* l2 = reinterpret_cast<const ulonglong2*>(l);
+    int r = 0;
+#pragma unroll 4
+    for (int j = 0; j < (m + 1) / 2; j++) {
+        const ulonglong2 y = l2[j];
+        r += (y.x > x) + (y.y > x);
+    }
+    return r;
+}
+
+// The first min(n, 4) keys of a list, zeros past them: one 32-byte load where
+// every list starts on such a boundary (wide), since four 8-byte loads of
+// lists that lie apart each take the load unit 32 cycles per warp.
+__device__ __forceinline__ void load4(const uint64_t* l, int n, bool wide, uint64_t (&v)[4]) {
+    if (wide) {
+        asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(l));
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) v[j] = j < n ? __ldcg(reinterpret_cast<const unsigned long long*>(l) + j) : 0ull;
+}
+
+// Appends the keys of keys[0..n) that reach T (none is 0) to surv.
+__device__ __forceinline__ void append_reaching(const uint64_t* keys, int n, uint64_t T, uint64_t* surv, int* cnt, int t0,
+                                                int nt) {
+#pragma unroll 1
+    for (int i = t0; i < n; i += nt) {
+        const uint64_t x = keys[i];
+        if (x != 0ull && x >= T) {
+            const int pos = atomicAdd(cnt, 1);
+            if (pos < kRankMax) surv[pos] = x;
+        }
+    }
+}
+
+// npb nodes per block: block r of a cluster merges the nodes r * npb ...
+template <int kPer>
+__global__ void __launch_bounds__(kMergeThreads) merge_select_kernel(const SelectArgs a, int cs, int npb) {
     pdl_trigger();
-    pdl_wait();
-    // dynamic: max(nV*k, W*k) keys, kRankMax survivors, 64 outputs, W*k candidate tokens
-    extern __shared__ uint64_t keys[];
+    constexpr int kNodes = kMergeThreads / kPer, kWarps = kPer / 32;
+    extern __shared__ __align__(16) uint64_t survs[];  // [nh][kRankMax] keys that reach the threshold
+    __shared__ __align__(16) uint64_t heads2[kNodes][kPer];  // list heads, or per-warp group maxima [kWarps][32]
+    __shared__ float redm2[kNodes][kWarps], redf2[kNodes][kWarps];
     __shared__ uint32_t hist[256];
     __shared__ int scal[4];
-    __shared__ uint64_t thr;
-    __shared__ float redf[32];
-    __shared__ float redm[32];
-    __shared__ int redi[32];
-    __shared__ int ticket;
-    const int cap = max(a.nV * a.klist, a.W * a.k);
-    uint64_t* surv = keys + cap;
-    uint64_t* top = surv + kRankMax;
-    int* ctok = reinterpret_cast<int*>(top + 64);
-
-    const int n = blockIdx.x, tid = threadIdx.x;
-    const int s = n / a.P, p = n % a.P;
-    // this node's partials are contiguous: part_ms[n][nV], part_key[n][nV][klist];
-    // they are loaded before the frontier size is known (rows past it hold
-    // stale but harmless data)
-    const int nk = a.nV * a.klist;
-    const uint64_t* blk = a.part_key + static_cast<size_t>(n) * part_stride(a.nV, a.klist);  // 16-byte aligned
-    const uint4* src = reinterpret_cast<const uint4*>(blk);
+    __shared__ int cnt2[kNodes];
+    __shared__ uint64_t thr2[kNodes];
+    const int nh = blockDim.x / kPer;  // nodes at once
+    const int fk = (a.P * a.k + 1) & ~1, stride = part_stride(a.nV, a.klist);
+    const int half = threadIdx.x / kPer, tid = threadIdx.x % kPer, lane = tid & 31, warp = tid >> 5;
+    uint64_t* surv = survs + half * kRankMax;
+    uint64_t* fkey = survs + nh * kRankMax;  // [P * k] block 0: the frontier's candidates, sorted per parent
+    const bool search = a.P <= kMergeSearchP;
+    int* ftok = reinterpret_cast<int*>(fkey + fk);  // [P * k] with `search`; else read from node_tok
+    uint64_t* heads = heads2[half];
+    const int rank = blockIdx.x % cs, s = blockIdx.x / cs;
+    const float2 none = make_float2(-INFINITY, 0.0f);
+    const bool wide = (a.klist & 3) == 0 && (reinterpret_cast<uintptr_t>(a.part_key) & 31u) == 0;
+    pdl_wait();
     const int prev_count = a.dep == 1 ? 1 : __ldcg(a.tree_count + s * a.L + a.dep - 2);
-    const uint64_t bound = a.gthr ? __ldcg(reinterpret_cast<const unsigned long long*>(a.gthr) + n) : 0ull;
-    float2 acc = make_float2(-INFINITY, 0.0f);
-    {
-        // every load of this thread is issued before the first use: one
-        // L2 round trip instead of one per loop iteration
-        constexpr int kBatch = 8;
-        float2 ms[2];
-#pragma unroll
-        for (int u = 0; u < 2; u++) {
-            const int r = tid + u * kSelThreads;
-            ms[u] = r < a.nV ? __ldcg(a.part_ms + static_cast<size_t>(n) * a.nV + r) : make_float2(-INFINITY, 0.0f);
-        }
-        for (int r = tid + 2 * kSelThreads; r < a.nV; r += kSelThreads)
-            acc = lse_merge(acc, __ldcg(a.part_ms + static_cast<size_t>(n) * a.nV + r));
-        for (int i0 = 0; i0 < nk / 2; i0 += kBatch * kSelThreads) {
-            uint4 v[kBatch];
-#pragma unroll
-            for (int u = 0; u < kBatch; u++) {
-                const int i = i0 + u * kSelThreads + tid;
-                if (i < nk / 2) v[u] = __ldcg(src + i);
-            }
-#pragma unroll
-            for (int u = 0; u < kBatch; u++) {
-                const int i = i0 + u * kSelThreads + tid;
-                if (i < nk / 2) reinterpret_cast<uint4*>(keys)[i] = v[u];
-            }
-        }
-        if ((nk & 1) && tid == 0) keys[nk - 1] = __ldcg(blk + nk - 1);
-        acc = lse_merge(acc, ms[0]);
-        acc = lse_merge(acc, ms[1]);
-    }
-
-    if (p < prev_count) {
-        // log-sum-exp of the node's scaled logits from the per-CTA partials
-        float m = warp_max(acc.x);
-        if ((tid & 31) == 0) redm[tid >> 5] = m;
-        __syncthreads();
-        float gm = -INFINITY;
-        for (int i = 0; i < kSelThreads / 32; i++) gm = fmaxf(gm, redm[i]);
-        const float part = acc.x == -INFINITY ? 0.0f : acc.y * __expf(acc.x - gm);
-        const float ssum = block_sum_float(part, redf);
-        const float lse = gm == -INFINITY ? -INFINITY : gm + logf(ssum);
-        // top-k over every CTA's (sorted) top-k list
-        topk_of_sorted_lists(keys, a.nV, a.klist, a.k, bound, top, surv, &thr, hist, scal);
-        for (int j = tid; j < a.k; j += kSelThreads) {
-            const uint64_t x = top[j];
-            const float z = key_val(x);
-            float lq = -INFINITY;
-            if (lse != -INFINITY && z != -INFINITY) lq = fminf(z - lse, 0.0f);
-            a.node_logq[static_cast<size_t>(n) * a.k + j] = lq;
-            a.node_tok[static_cast<size_t>(n) * a.k + j] = static_cast<int>(key_idx(x));
-        }
+    const uint32_t fk0 = smem_u32(fkey), ft0 = smem_u32(ftok);
+#pragma unroll 1
+    for (int it = 0; it * nh < npb; it++) {
+        const int p = rank * npb + it * nh + half, n = s * a.P + p;
+        const bool mine = it * nh + half < npb && p < a.P;
+        // the loads of one round trip: partials, the first keys of this
+        // thread's list, the bound, the parent's score
+        const float2* ms = a.part_ms + static_cast<size_t>(n) * a.nV;
+        const uint64_t* lists = a.part_key + static_cast<size_t>(n) * stride;
+        const float2 m0 = mine && tid < a.nV ? __ldcg(ms + tid) : none;
+        const float2 m1 = mine && tid + kPer < a.nV ? __ldcg(ms + tid + kPer) : none;
+        uint64_t v[4] = {0ull, 0ull, 0ull, 0ull};
+        if (mine && tid < a.nV) load4(lists + tid * a.klist, a.klist, wide, v);
+        const uint64_t bound =
+            a.gthr && mine ? __ldcg(reinterpret_cast<const unsigned long long*>(a.gthr) + n) : 0ull;
+        const float ps = a.dep == 1 || !mine
+                             ? 0.0f
+                             : __ldcg(a.tree_score + (static_cast<size_t>(s) * a.L + a.dep - 2) * a.W + p);
+        const float2 acc = lse_merge(m0, m1);
+        const float wm = warp_max(acc.x);
+        if (lane == 0) redm2[half][warp] = wm;
         if (tid == 0) {
-            a.node_lse[n] = lse;
-            if (a.lse_hist) a.lse_hist[static_cast<size_t>(n) * a.lse_hist_stride] = lse;
+            cnt2[half] = 0;
+            thr2[half] = 0ull;
+        }
+        // threshold: a key that at least k keys reach.  Up to kGroupMaxK: the
+        // heads are dealt into 2^q >= k groups, each of whose maxima reaches
+        // the least of them; above: the k-th largest head.  (Lists past kPer,
+        // which only candidate sets of more than 512 tokens have, are left out.)
+        const bool groups = a.k <= kGroupMaxK;
+        const int q2 = a.k <= 1 ? 1 : 1 << (32 - __clz(a.k - 1));
+        uint64_t g = v[0];
+        if (groups) {
+#pragma unroll 1
+            for (int o = 16; o >= q2; o >>= 1) {
+                const uint64_t y = shfl_xor_u64(g, o);
+                g = y > g ? y : g;
+            }
+        }
+        heads[tid] = g;  // groups: of warp `warp`, group lane mod q2
+        __syncthreads();
+        const float gm = warp_max(redm2[half][lane % kWarps]);
+        float part = acc.x == -INFINITY ? 0.0f : acc.y * __expf(acc.x - gm);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
+        if (lane == 0) redf2[half][warp] = part;
+        uint64_t T = 0ull;
+        if (groups) {
+#pragma unroll 1
+            for (int w = 0; w < kWarps; w++) {
+                const uint64_t y = heads[w * 32 + (lane & (q2 - 1))];
+                T = y > T ? y : T;
+            }
+#pragma unroll 1
+            for (int o = q2 >> 1; o > 0; o >>= 1) {
+                const uint64_t y = shfl_xor_u64(T, o);
+                T = y < T ? y : T;
+            }
+        } else {
+            const int nl = min(a.nV, kPer);
+            if (v[0] != 0ull && count_above(heads, nl, v[0]) == a.k - 1) thr2[half] = v[0];
+            __syncthreads();
+            T = thr2[half];
+        }
+        T = T > bound ? T : bound;
+        {
+            auto take = [&](uint64_t x) -> bool {
+                if (x == 0ull || x < T) return false;
+                const int pos = atomicAdd(&cnt2[half], 1);
+                if (pos < kRankMax) surv[pos] = x;
+                return true;
+            };
+            bool more = take(v[0]) && take(v[1]) && take(v[2]) && take(v[3]);
+#pragma unroll 1
+            for (int r = tid, j = 4; mine && r < a.nV; r += kPer, j = 0, more = true) {
+#pragma unroll 1
+                for (; more && j < a.klist; j += 4) {
+                    load4(lists + r * a.klist + j, a.klist - j, wide, v);
+                    more = take(v[0]) && take(v[1]) && take(v[2]) && take(v[3]);
+                }
+            }
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int h = 0; h < nh; h++) {
+            if (cnt2[h] > kRankMax) {
+                radix_survivors(a.part_key + static_cast<size_t>(n + h - half) * stride, a.nV * a.klist, a.k,
+                                survs + h * kRankMax, hist, scal);
+                if (threadIdx.x == 0) cnt2[h] = a.k;
+                __syncthreads();
+            }
+        }
+        const int m = cnt2[half];
+        if ((m & 1) && tid == 0) surv[m] = 0ull;  // (an odd m leaves room)
+        float ssum = 0.0f;
+#pragma unroll
+        for (int i = 0; i < kWarps; i++) ssum += redf2[half][i];  // (in warp order)
+        const float lse = gm == -INFINITY ? -INFINITY : gm + logf(ssum);
+        const bool live = mine && p < prev_count;
+        if (mine && tid == 0) {
+            a.node_lse[n] = live ? lse : -INFINITY;
+            if (a.lse_hist && live) a.lse_hist[static_cast<size_t>(n) * a.lse_hist_stride] = lse;
+        }
+        __syncthreads();
+        if (live) {
+#pragma unroll 1
+            for (int i = tid; i < m; i += kPer) {
+                const uint64_t x = surv[i];
+                const int j = count_above(surv, m, x);
+                if (j >= a.k) continue;
+                const float z = key_val(x);
+                const int tok = static_cast<int>(key_idx(x));
+                const float lq = (lse != -INFINITY && z != -INFINITY) ? fminf(z - lse, 0.0f) : -INFINITY;
+                a.node_logq[static_cast<size_t>(n) * a.k + j] = lq;
+                a.node_tok[static_cast<size_t>(n) * a.k + j] = tok;
+                const float sc = (ps + lq) + a.beta;  // Eq. 5, one more depth
+                const int c = p * a.k + j;
+                st_cluster_u64(fk0 + c * 8, 0, sc > -INFINITY ? make_key(sc, static_cast<uint32_t>(c)) : 0ull);
+                if (search) st_cluster_s32(ft0 + c * 4, 0, tok);
+            }
+        } else if (mine && tid < a.k) {
+            a.node_logq[static_cast<size_t>(n) * a.k + tid] = -INFINITY;
+            a.node_tok[static_cast<size_t>(n) * a.k + tid] = -1;
+        }
+        __syncthreads();  // this node's buffers are free for the next
+    }
+    cluster_sync_all();
+    if (rank != 0) return;
+    // block 0: the top W of the candidates (p, j), sorted for every parent p
+    const int t = threadIdx.x, nt = blockDim.x;
+    const int ncand = prev_count * a.k;
+    const size_t tb = (static_cast<size_t>(s) * a.L + a.dep - 1) * a.W;
+    auto keep = [&](uint64_t x, int r) {
+        const int c = static_cast<int>(key_idx(x));
+        if (r >= a.W || !bounds_check(a.status, c < ncand)) return;
+        const int pp = c / a.k, tok = search ? ftok[c] : __ldcg(a.node_tok + static_cast<size_t>(s) * a.P * a.k + c);
+        a.tree_tok[tb + r] = tok;
+        a.tree_parent[tb + r] = a.dep == 1 ? -1 : pp;
+        a.tree_score[tb + r] = key_val(x);
+        if (r < a.Pn) {
+            a.child_prow[s * a.Pn + r] = s * a.P + pp;
+            a.child_tok[s * a.Pn + r] = tok;
+        }
+    };
+    int nvalid = 0;
+    if (search) {
+#pragma unroll 1
+        for (int c0 = 0; c0 < ncand; c0 += nt) {
+            const uint64_t x = c0 + t < ncand ? fkey[c0 + t] : 0ull;
+            nvalid += __syncthreads_count(x != 0ull);
+            if (x == 0ull) continue;
+            int r = 0;
+#pragma unroll 1
+            for (int o = 0; o < prev_count; o++) r += count_greater(fkey + o * a.k, a.k, x);
+            keep(x, r);
         }
     } else {
-        for (int j = tid; j < a.k; j += kSelThreads) {
-            a.node_logq[static_cast<size_t>(n) * a.k + j] = -INFINITY;
-            a.node_tok[static_cast<size_t>(n) * a.k + j] = -1;
+        // (nt >= P) at least W candidates reach the W-th largest list head
+        if (t == 0) {
+            cnt2[0] = 0;
+            thr2[0] = 0ull;
         }
-        if (tid == 0) a.node_lse[n] = -INFINITY;
+        uint64_t* fh = heads2[0];
+        if (t < prev_count + 1) fh[t] = t < prev_count ? fkey[t * a.k] : 0ull;
+        __syncthreads();
+        if (t < prev_count && fh[t] != 0ull && count_above(fh, prev_count, fh[t]) == a.W - 1) thr2[0] = fh[t];
+        for (int c0 = 0; c0 < ncand; c0 += nt) nvalid += __syncthreads_count(c0 + t < ncand && fkey[c0 + t] != 0ull);
+        append_reaching(fkey, ncand, thr2[0], survs, &cnt2[0], t, nt);
+        __syncthreads();
+        int m = cnt2[0];
+        if (m > kRankMax) {
+            m = min(a.W, nvalid);
+            radix_survivors(fkey, ncand, m, survs, hist, scal);
+        }
+        if ((m & 1) && t == 0) survs[m] = 0ull;
+        __syncthreads();
+        if (t < m) keep(survs[t], count_above(survs, m, survs[t]));
+        if (t + nt < m) keep(survs[t + nt], count_above(survs, m, survs[t + nt]));
     }
-
-    // The last node block of this sequence selects S_d (no block ever waits).
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) ticket = atomicAdd(&a.seq_ticket[s], 1);
-    __syncthreads();
-    if (ticket != a.P - 1) return;
-    __threadfence();
-    if (tid == 0) a.seq_ticket[s] = 0;
-
-    select_frontier(a, s, prev_count, keys, ctok, surv, top, &thr, hist, scal, redi);
+    const int cnt = min(a.W, nvalid);
+#pragma unroll 1
+    for (int r = cnt + t; r < a.W; r += nt) {
+        a.tree_tok[tb + r] = -1;
+        a.tree_parent[tb + r] = -1;
+        a.tree_score[tb + r] = -INFINITY;
+        if (r < a.Pn) {
+            a.child_prow[s * a.Pn + r] = -1;
+            a.child_tok[s * a.Pn + r] = 0;
+        }
+    }
+    if (t == 0) a.tree_count[s * a.L + a.dep - 1] = cnt;
 }
 
 // Only the log-sum-exp of each node (the same arithmetic), of the nodes with
@@ -338,15 +537,41 @@ __global__ void __launch_bounds__(NT) residual_norm_kernel(int d, int S, int Nc,
 
 bool pdl_enabled() { return true; }
 
-int merge_select_smem(int nV, int klist, int k, int W) {
-    return (max(nV * klist, W * k) + kRankMax + 64) * 8 + W * k * 4;
+// Launch shape: 256 threads per node up to 256 vocabulary ranges, else 512.
+// Two nodes per block, so that a cluster is small (it starts when all of its
+// blocks fit on one GPC at once), four where more than 16 blocks were needed.
+// Measured on GB300 (µs per round): 16 nodes, k = 16: 3422 with one or two
+// nodes per block, 3441 with four.
+struct MergePlan {
+    int per, nh, cs, npb, smem;
+};
+static MergePlan merge_plan(int P, int nV, int k) {
+    MergePlan m;
+    m.per = nV <= 256 ? 256 : 512;
+    m.nh = std::min({P, P <= 2 * kMergeCluster ? 2 : 4, kMergeThreads / m.per});
+    const int cs = std::min((P + m.nh - 1) / m.nh, kMergeCluster);
+    m.npb = (P + cs - 1) / cs;
+    m.cs = (P + m.npb - 1) / m.npb;
+    m.smem = (m.nh * kRankMax + ((P * k + 1) & ~1)) * 8 + (P <= kMergeSearchP ? P * k * 4 : 0);
+    return m;
 }
 
-cudaError_t select_set_smem_limits() { return set_max_dynamic_smem(reinterpret_cast<const void*>(merge_select_kernel)); }
+int merge_select_smem(int P, int nV, int k) { return merge_plan(P, nV, k).smem; }
+
+cudaError_t select_set_smem_limits() {
+    cudaError_t e = cudaSuccess;
+    for (const void* fn : {reinterpret_cast<const void*>(merge_select_kernel<256>),
+                           reinterpret_cast<const void*>(merge_select_kernel<512>)}) {
+        if (e == cudaSuccess) e = set_max_dynamic_smem(fn);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
+    return e;
+}
 
 cudaError_t launch_merge_select(const SelectArgs& a, cudaStream_t st) {
-    const int smem = merge_select_smem(a.nV, a.klist, a.k, a.W);
-    return launch_pdl(merge_select_kernel, dim3(a.N), dim3(kSelThreads), smem, st, a);
+    const MergePlan m = merge_plan(a.P, a.nV, a.k);
+    return launch_pdl_cluster(m.per == 256 ? merge_select_kernel<256> : merge_select_kernel<512>,
+                              dim3(a.nseq * m.cs), dim3(m.nh * m.per), m.smem, st, m.cs, a, m.cs, m.npb);
 }
 
 cudaError_t launch_merge_lse(const float2* part_ms, int N, int nV, const int* row_ent, float* lse, cudaStream_t st) {
