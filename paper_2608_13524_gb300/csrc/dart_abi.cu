@@ -118,8 +118,6 @@ struct dart_handle {
     uint64_t* gthr;  // [L][kNPadMax] cross-CTA top-k bounds of every depth, zeroed per round
     float* bound_y;     // [kNPadMax][kBoundR] seed scores less their error bounds (topk_bound)
     int* cand_tok;   // [nseq][L][cand_k] candidate sets C_d (cand_k > 0)
-    float* cand_scratch;  // candidate scoring partial dot products
-    int* cand_ticket;     // [nseq][ceil(cand_k/8)]
     uint64_t* cand_part;  // [nseq * L][slices][cand_k] per-slice top keys of the candidate selection
     int* cand_rticket;    // [nseq * L] slices finished per row
     float* Qtab;          // [V][d] fp32: Q[t] = W_i[:, d:2d] . E[t] (split first head layer), or null
@@ -665,12 +663,7 @@ int alloc_workspace(dart_handle* h) {
         DART_ALLOC(h->sh_ticket, ns * M)
     }
     if (c.cand_k > 0) {
-        size_t scr = 1;
-        for (int dep = 1; dep <= c.L; dep++)
-            scr = std::max(scr, static_cast<size_t>(h->plans[dep].cand_ds) * h->plans[dep].N * c.cand_k);
         DART_ALLOC(h->cand_tok, static_cast<size_t>(c.nseq) * c.L * c.cand_k)
-        DART_ALLOC(h->cand_scratch, scr)
-        DART_ALLOC(h->cand_ticket, static_cast<size_t>(c.nseq) * ((c.cand_k + 7) / 8))
         DART_ALLOC(h->cand_part, static_cast<size_t>(c.nseq) * c.L *
                                      cand_topk_slices(c.V, c.cand_k, c.nseq * c.L, h->num_sms) * c.cand_k)
         DART_ALLOC(h->cand_rticket, static_cast<size_t>(c.nseq) * c.L)
@@ -705,10 +698,9 @@ int alloc_workspace(dart_handle* h) {
     if (select_set_smem_limits() != cudaSuccess) return DART_ERR_CUDA;
     if (c.cand_k > 0) {
         for (int dep = 1; dep <= c.L; dep++)
-            if (cand_score_smem(h->plans[dep].P, c.d, h->plans[dep].cand_ds) > h->smem_optin - 1024)
+            if (h->plans[dep].P * (c.d / h->plans[dep].cand_ds) * 4 > h->smem_optin - 1024)
                 return DART_ERR_UNSUPPORTED;
-        if (cudaMemset(h->cand_ticket, 0, c.nseq * ((c.cand_k + 7) / 8) * sizeof(int)) != cudaSuccess ||
-            cudaMemset(h->cand_rticket, 0, static_cast<size_t>(c.nseq) * c.L * sizeof(int)) != cudaSuccess)
+        if (cudaMemset(h->cand_rticket, 0, static_cast<size_t>(c.nseq) * c.L * sizeof(int)) != cudaSuccess)
             return DART_ERR_CUDA;
     }
     if ((c.cand_k > 0 || c.variants) && cand_set_smem_limits() != cudaSuccess) return DART_ERR_CUDA;
@@ -953,8 +945,6 @@ int enqueue_depth(dart_handle* h, const dart_config& c, const std::vector<DepthP
         ca.part_ms = h->part_ms;
         ca.part_key = h->part_key;
         ca.DS = p.cand_ds;
-        ca.scratch = h->cand_scratch;
-        ca.ticket = h->cand_ticket;
         pi = prof_begin(h, kCandScore, st);
         e = launch_cand_score(ca, st);
     } else {

@@ -233,8 +233,6 @@ struct CandArgs {
     float2* part_ms;            // [nseq*P][K]  (z, 1)
     uint64_t* part_key;         // [nseq*P][part_stride(K, 1)]  key(z, token)
     int DS;                     // d slices (blocks per candidate group), see cand_score_slices
-    float* scratch;             // [DS][nseq*P][K] partial dot products
-    int* ticket;                // [nseq][ceil(K/8)] zero between launches
 };
 // S = cand_topk_slices(V, K, rows, SMs) blocks per row; part: [rows][S][K]
 // keys, ticket: [rows] ints, zero before the first launch (every launch
@@ -251,7 +249,6 @@ int cand_topk_slices(int V, int K, int rows, int num_sms);
 cudaError_t launch_cand_score(const CandArgs& a, cudaStream_t st);
 int cand_topk_smem(int K);
 int cand_score_slices(int P, int d, int nseq, int K, int max_smem);  // 0: does not fit
-int cand_score_smem(int P, int d, int DS);
 cudaError_t cand_set_smem_limits();    // the device maximum for both kernels
 
 struct EmitArgs {
