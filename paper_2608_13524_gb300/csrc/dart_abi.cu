@@ -520,6 +520,19 @@ int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, st
                         g->S = std::max(1, std::min(g->KB, cap / tiles_mg));
                     }
                 }
+                // A grid of at most one CTA per SM: all of an SM's shared
+                // memory for its pipeline (the loads in flight, not the
+                // tensor cores, bound a CTA that walks a long k range).
+                // Measured on GB300, 256 nodes, d = 4096 (128 CTAs of 64
+                // k-blocks): 3 stages 34.1 us per GEMM and 1289 us per
+                // round of 8 x 32 nodes with K = 64, 7 stages 30.0 and 1179.
+                for (GemmArgs* g : {&p.g1, &p.g2}) {
+                    int& sm = g == &p.g1 ? p.g1_smem : p.g2_smem;
+                    const int sbg = tc_stage_bytes(g->NG);
+                    if (g->MT * g->G * g->S <= h->num_sms)
+                        g->stages = std::min(tc_stages(h->smem_optin, sbg, gemm_tc_fixed_smem(16)), 8);
+                    sm = gemm_tc_fixed_smem(g->stages) + g->stages * sbg;
+                }
                 p.g1.mode = cluster1 ? (p.split ? kGemmSum : kGemmSiluSplit) : kGemmPartials;
                 p.g2.mode = cluster ? kGemmSum : kGemmPartials;
                 p.g1.a_tiled_kb = h->wtiled ? h->Kwi / kBlockK : 0;

@@ -269,13 +269,11 @@ template <int NG>
 constexpr int acc_stride() {
     return 2 * NG < 32 ? 32 : 2 * NG;
 }
+// TMEM columns of a GEMM CTA: one tile, hence one accumulator (a power of two
+// of at least 32 columns).
 template <int NG>
 constexpr int tmem_cols() {
-    return 2 * acc_stride<NG>() <= 32 ? 32
-                                      : (2 * acc_stride<NG>() <= 64 ? 64
-                                                                    : (2 * acc_stride<NG>() <= 128
-                                                                           ? 128
-                                                                           : (2 * acc_stride<NG>() <= 256 ? 256 : 512)));
+    return acc_stride<NG>();
 }
 
 // Accumulators of the LM-head (a ring in TMEM): with 64-node groups four,
@@ -476,8 +474,9 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
 //                   order (deterministic) and writes outL = hi/lo bf16 split
 //                   of SiLU(sum) (input of W_o), or out = sum in fp32.
 
+// (two CTAs per SM: at most 56 registers per thread)
 template <int NG>
-__global__ void __launch_bounds__(threads<NG>(), 1)
+__global__ void __launch_bounds__(threads<NG>(), 2)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const GemmArgs a) {
     extern __shared__ uint8_t smem_raw[];
@@ -551,32 +550,46 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
     if (a.mode == kGemmPartials) return;  // launched without clusters
     cluster_sync_all();  // every split's tile is staged
     {
+        // units of 4 rows (M is a multiple of 64: a unit is inside or outside whole)
         const int S = a.S;
         const uint32_t r = cluster_ctarank();
-        const int R = (kTileM + S - 1) / S;
-        const int nthr = threads<NG>();
+        const int u0 = static_cast<int>(r) * (kTileM / 4) / S, nu = (static_cast<int>(r) + 1) * (kTileM / 4) / S - u0;
         const uint32_t base = smem_u32(stage_tile);
-        for (int idx = threadIdx.x; idx < R * NG; idx += nthr) {
-            const int nl = idx / R, row = static_cast<int>(r) * R + idx % R;
+#pragma unroll 1
+        for (int idx = threadIdx.x; idx < nu * NG; idx += threads<NG>()) {
+            const int nl = idx / nu, row = (u0 + idx % nu) * 4;
             const int m = w.row0 + row, n = g_c * NG + nl;
-            if (row >= kTileM || m >= a.M || n >= a.N) continue;
+            if (m >= a.M || n >= a.N) continue;
             const uint32_t off = base + static_cast<uint32_t>((nl * kTileM + row) * 4);
-            float v[kMaxClusterK];
+            float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 1
+            for (int q0 = 0; q0 < S; q0 += 4) {  // four loads in flight
+                float4 v[4];
 #pragma unroll
-            for (int q = 0; q < kMaxClusterK; q++) v[q] = q < S ? ld_cluster_f32(off, static_cast<uint32_t>(q)) : 0.0f;
-            float acc = 0.0f;
+                for (int q = 0; q < 4; q++)
+                    if (q0 + q < S) v[q] = ld_cluster_f32x4(off, static_cast<uint32_t>(q0 + q));
 #pragma unroll
-            for (int q = 0; q < kMaxClusterK; q++)
-                if (q < S) acc += v[q];
+                for (int q = 0; q < 4; q++) {
+                    if (q0 + q < S) {
+                        acc.x += v[q].x;
+                        acc.y += v[q].y;
+                        acc.z += v[q].z;
+                        acc.w += v[q].w;
+                    }
+                }
+            }
             const size_t o = static_cast<size_t>(n) * a.M + m;
             if (a.mode == kGemmSiluSplit) {
-                const float act = acc / (1.0f + expf(-acc));
-                __nv_bfloat16 hi, lo;
-                split_bf16(act, hi, lo);
-                a.outL[o] = hi;
-                a.outL[static_cast<size_t>(a.bhalf) * a.M + o] = lo;
+                const float act[4] = {acc.x / (1.0f + expf(-acc.x)), acc.y / (1.0f + expf(-acc.y)),
+                                      acc.z / (1.0f + expf(-acc.z)), acc.w / (1.0f + expf(-acc.w))};
+                __align__(8) __nv_bfloat16 hi[4], lo[4];
+#pragma unroll
+                for (int e = 0; e < 4; e++) split_bf16(act[e], hi[e], lo[e]);
+                *reinterpret_cast<uint2*>(a.outL + o) = *reinterpret_cast<const uint2*>(hi);
+                *reinterpret_cast<uint2*>(a.outL + static_cast<size_t>(a.bhalf) * a.M + o) =
+                    *reinterpret_cast<const uint2*>(lo);
             } else {
-                a.out[o] = acc;
+                *reinterpret_cast<float4*>(a.out + o) = acc;
             }
         }
     }
