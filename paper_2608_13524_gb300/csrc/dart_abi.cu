@@ -68,6 +68,7 @@ int ng_index(int NG) { return NG == 16 ? 0 : (NG == 32 ? 1 : (NG == 64 ? 2 : 3))
 
 struct DepthPlan {
     int N, P, NG, G, nV, stages, smem;  // LM-head scoring
+    int pair;                            // LM-head: CTA pairs
     int l2pf;                            // LM-head: E tiles per CTA prefetched into L2 before its wait
     int epf;                             // of those and the stages, how many the previous depth prefetches early
     int bound;                           // seed rows per sequence of the seed pass before this depth's LM-head (0: none)
@@ -392,6 +393,7 @@ int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, st
             p.nV = lp.nV;
             p.stages = lp.stages;
             p.smem = lp.smem;
+            p.pair = lp.pair ? 1 : 0;
             // One group of <= 16 nodes: every CTA streams its own slice of
             // E and the launch is HBM-bound.  Besides the stages it loads
             // before waiting on the previous kernel (which is latency-bound
@@ -849,6 +851,7 @@ LmheadArgs lmhead_args(const dart_handle* h, const dart_config& c, const DepthPl
     la.dlog_seq_stride = static_cast<long long>(c.L) * c.V;
     la.bhalf = kNPadMax;
     la.stages = p.stages;
+    la.pair = p.pair;
     la.l2pf = p.l2pf;
     la.part_ms = h->part_ms;
     la.part_key = h->part_key;

@@ -40,7 +40,7 @@ constexpr int kNPadMax = 256;       // max nodes per depth (nseq * W)
 constexpr int kTileM = 128;         // MMA M: vocabulary rows / output features per tile
 constexpr int kBlockK = 64;         // bf16 elements per 128-byte swizzled row
 constexpr int kCandCap = 128;       // per-node candidate slots per tile (one tile worth)
-constexpr int kCandCapLarge = 32;   // slots per node for 128-node groups (overflow: more merge rounds)
+constexpr int kCandCapLarge = 32;   // slots per node for 64-node groups, twice those of 128 (overflow: more merge rounds)
 constexpr int kEpiBarrier = 1;      // named barrier id used by the epilogue warps
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -214,6 +214,57 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
                      smem_u32(bar))
                  : "memory");
 }
+// ---- CTA pairs (cta_group::2): the two CTAs of a cluster of two work on one
+// MMA of M = 256; each holds its own 128 rows of A and of the accumulator and
+// half of B's rows in its shared memory; the even CTA (the leader) issues.
+
+// Shared-memory address of CTA `rank` of the cluster at the offset of the local address.
+__device__ __forceinline__ uint32_t mapa_u32(uint32_t local, uint32_t rank) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+    return remote;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t remote_bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote_bar) : "memory");
+}
+// 2-D tiled bulk copy into this CTA, completing on a barrier of the pair (a
+// shared::cluster address).
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, uint32_t bar, int x, int y,
+                                                 uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint"
+        " [%0], [%1, {%3, %4}], [%2], %5;" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "l"(policy)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* slot, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(ncols)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_relinquish_pair() {
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void tc_mma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                 uint32_t accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// Arrives once on the barrier at this offset in both CTAs of the pair when
+// every tcgen05 op issued so far by this thread is done.
+__device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"(static_cast<uint16_t>(3))
+        : "memory");
+}
+
 // 32 TMEM lanes x 16 consecutive 32-bit columns: thread i of the warp gets lane
 // (warp's lane quarter + i), columns [col, col+16).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {

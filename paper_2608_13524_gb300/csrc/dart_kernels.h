@@ -95,6 +95,7 @@ struct LmheadArgs {
     const float* E32;     // fp32 table [V][d]   (fp32 kernel)
     uint64_t* gthr;       // [N] cross-CTA top-k bounds, zero before the launch (may be null)
     int e_tiled;          // the E tensor map is over the tiled copy (launch_retile), not [V][d]
+    int pair;             // launch as CTA pairs (LmheadPlan)
     int DS;               // fp32 kernel: blocks (one cluster) sharing a vocabulary range, each a slice of d
     // optional (null: unused)
     const int* dlog_row;  // [N / P] drafter row of each sequence's nodes (replaces dlog_row_off / V)
@@ -175,6 +176,7 @@ cudaError_t launch_lmhead_l2_prefetch(const CUtensorMap* tmE, int tiles, int nV,
 // plan fits the device.
 struct LmheadPlan {
     int NG, G, nV, stages, smem;
+    bool pair;  // two neighbouring vocabulary ranges as a CTA pair
 };
 bool plan_lmhead_tc(int N, int V, int d, int k, int num_sms, int smem_optin, int ctas_per_sm_pref, bool e_tiled,
                     LmheadPlan* out);

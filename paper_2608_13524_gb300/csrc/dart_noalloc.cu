@@ -195,6 +195,7 @@ extern "C" int dart_expand_root_noalloc(const dart_config* cfg, const void* E, c
     la.dlog_row_off = 0;
     la.bhalf = kBhalfNoAlloc;
     la.stages = lp.stages;
+    la.pair = lp.pair ? 1 : 0;
     la.part_ms = part_ms;
     la.part_key = part_key;
     la.status = status;

@@ -48,10 +48,12 @@ constexpr int epi_chunks() {
 // starting bound of the filter (seed pass before the launch), after which
 // a tile rarely offers more than a few logits per node.  Measured on GB300
 // at 64 nodes, k = 64 (µs per round, same box): 128 slots 3042, 64 slots
-// 2806, 32 slots 2706 with the bound; without it 32 slots cost +6 %.
+// 2806, 32 slots 2706 with the bound; without it 32 slots cost +6 %.  128-node
+// groups keep 16, which makes room for a fifth stage (389 instead of 403 µs
+// per launch at 256 nodes; 8 slots change nothing more).
 template <int NG>
 constexpr int lm_cand_cap() {
-    return NG >= 64 ? kCandCapLarge : kCandCap;
+    return NG > 64 ? kCandCapLarge / 2 : NG == 64 ? kCandCapLarge : kCandCap;
 }
 template <int NG>
 constexpr int threads() {
@@ -204,6 +206,121 @@ __device__ __forceinline__ void mma_issuer(const Work& w, uint8_t* ring, int sta
     }
 }
 
+// ---- the same roles for a CTA pair (lmhead_pair_kernel, gemm_pair_kernel)
+//
+// Each CTA loads its own A tile (128 rows) and one half of the group's B
+// rows: the leader the hi rows, its peer the lo rows.  A stage is full when
+// all four copies have completed on the leader's barrier; it is empty when
+// the leader's commit has arrived in both CTAs.
+
+template <int NG>
+struct PairLayout {
+    static constexpr int kStage = kATileBytes + NG * 128;
+};
+
+template <int NG>
+__device__ __forceinline__ void producer_pair(const CUtensorMap* tmA, const CUtensorMap* tmB, const Work& w,
+                                              uint32_t rank, int bhalf, uint8_t* ring, int stages, uint64_t* full,
+                                              uint64_t* empty, volatile int* abort, int* status) {
+    const uint64_t pol_a = l2_policy_evict_first();  // streamed once
+    const uint64_t pol_b = l2_policy_evict_last();   // re-read by every tile
+    const int kbs = w.kb1 - w.kb0;
+    const uint32_t total = static_cast<uint32_t>(w.ntiles * kbs);
+    const uint32_t pre = total < static_cast<uint32_t>(stages) ? total : static_cast<uint32_t>(stages);
+    const int brow = w.brow + (rank ? bhalf : 0);
+    auto load_a = [&](uint32_t f, uint32_t st) {
+        const int i = static_cast<int>(f) / kbs, kb = w.kb0 + static_cast<int>(f) % kbs;
+        tma_load_2d_pair(ring + st * PairLayout<NG>::kStage, tmA, mapa_u32(smem_u32(&full[st]), 0), a_x(w, kb),
+                         a_y(w, i, kb), pol_a);
+    };
+    auto load_b = [&](uint32_t f, uint32_t st) {
+        tma_load_2d_pair(ring + st * PairLayout<NG>::kStage + kATileBytes, tmB, mapa_u32(smem_u32(&full[st]), 0),
+                         (w.kb0 + static_cast<int>(f) % kbs) * kBlockK, brow, pol_b);
+    };
+    // (as in `producer`: A does not depend on an earlier kernel, B does)
+    for (uint32_t f = 0; f < pre; f++) {
+        if (rank == 0) mbar_arrive_expect_tx(&full[f], 2 * PairLayout<NG>::kStage);
+        load_a(f, f);
+    }
+    pdl_wait();
+    for (uint32_t f = 0; f < pre; f++) load_b(f, f);
+    uint32_t stage = pre % stages, phase = (pre / stages) & 1u, fills = pre;
+    bool ok = true;
+    for (uint32_t f = pre; f < total; f++) {
+        if (!mbar_wait(&empty[stage], phase ^ 1u, abort)) {
+            record_timeout(status, abort);
+            ok = false;
+            break;
+        }
+        if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * PairLayout<NG>::kStage);
+        load_a(f, stage);
+        load_b(f, stage);
+        fills++;
+        if (++stage == static_cast<uint32_t>(stages)) {
+            stage = 0;
+            phase ^= 1u;
+        }
+    }
+    if (!ok) {
+        // copies still in flight must land before the pair leaves: the
+        // leader's barriers track both CTAs'; the peer, which cannot wait on
+        // them, stays a millisecond, far longer than a copy takes
+        if (rank == 0) {
+            const uint32_t first = fills > static_cast<uint32_t>(stages) ? fills - stages : 0;
+            for (uint32_t f = first; f < fills; f++) drain_wait(&full[f % stages], (f / stages) & 1u);
+        } else {
+            const unsigned long long t0 = globaltimer_ns();
+            while (globaltimer_ns() - t0 < 1000000ull) {
+            }
+        }
+    }
+}
+
+// One thread of the leader.
+template <int NG>
+__device__ __forceinline__ void mma_issuer_pair(const Work& w, uint8_t* ring, int stages, uint64_t* full,
+                                                uint64_t* empty, uint64_t* tfull, uint64_t* tempty, uint64_t* tdown,
+                                                uint32_t tmem_base, int acc_stride, volatile int* abort, int* status,
+                                                int nacc) {
+    constexpr uint32_t idesc = idesc_bf16_f32(2 * kTileM, 2 * NG);
+    uint32_t stage = 0, phase = 0;
+    bool ok = true;
+    for (int i = 0; i < w.ntiles && ok; i++) {
+        const int acc = i % nacc;
+        if (!mbar_wait(&tempty[acc], ((i / nacc) & 1) ^ 1u, abort)) {
+            record_timeout(status, abort);
+            ok = false;
+            break;
+        }
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + acc * acc_stride;
+        for (int kb = w.kb0; kb < w.kb1; kb++) {
+            if (!mbar_wait(&full[stage], phase, abort)) {
+                record_timeout(status, abort);
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t a = smem_u32(ring + stage * PairLayout<NG>::kStage);
+            const uint32_t hb = a + kATileBytes;
+#pragma unroll
+            for (int kk = 0; kk < kBlockK / 16; kk++)
+                tc_mma_bf16_pair(d_tmem, sdesc_sw128(a + kk * 32), sdesc_sw128(hb + kk * 32), idesc,
+                                 (kb > w.kb0 || kk > 0) ? 1u : 0u);
+            tc_commit_pair(&empty[stage]);
+            if (++stage == static_cast<uint32_t>(stages)) {
+                stage = 0;
+                phase ^= 1u;
+            }
+        }
+        if (ok) tc_commit_pair(&tfull[acc]);
+    }
+    if (!ok) {
+        tc_commit_pair(tdown);
+        drain_wait(tdown, 0);
+    }
+}
+
 struct Smem {
     uint8_t* ring;
     uint64_t *full, *empty, *tfull, *tempty, *tdown;
@@ -211,12 +328,12 @@ struct Smem {
     uint8_t* tail;
 };
 
-template <int NG>
+template <int NG, bool kPair = false>
 __device__ __forceinline__ Smem carve(uint8_t* raw, int stages, int nacc = 2) {
     Smem s;
     const uint32_t off = (1024u - (smem_u32(raw) & 1023u)) & 1023u;
     s.ring = raw + off;
-    s.full = reinterpret_cast<uint64_t*>(s.ring + stages * Layout<NG>::kStage);
+    s.full = reinterpret_cast<uint64_t*>(s.ring + stages * (kPair ? PairLayout<NG>::kStage : Layout<NG>::kStage));
     s.empty = s.full + stages;
     s.tfull = s.empty + stages;
     s.tempty = s.tfull + nacc;
@@ -226,7 +343,7 @@ __device__ __forceinline__ Smem carve(uint8_t* raw, int stages, int nacc = 2) {
     return s;
 }
 
-template <int NG>
+template <int NG, bool kPair = false>
 __device__ __forceinline__ uint32_t setup(const Smem& s, int stages, int ncols, int nacc = 2) {
     constexpr int kEpi = epi_threads<NG>();
     const int warp = threadIdx.x >> 5;
@@ -237,7 +354,7 @@ __device__ __forceinline__ uint32_t setup(const Smem& s, int stages, int ncols, 
         }
         for (int i = 0; i < nacc; i++) {
             mbar_init(&s.tfull[i], 1);
-            mbar_init(&s.tempty[i], kEpi);
+            mbar_init(&s.tempty[i], kPair ? 2 * kEpi / 32 : kEpi);  // pairs: a lane of every warp of both CTAs
         }
         mbar_init(s.tdown, 1);
         s.misc[1] = 0;
@@ -245,22 +362,31 @@ __device__ __forceinline__ uint32_t setup(const Smem& s, int stages, int ncols, 
         fence_mbar_init();
     }
     if (warp == 1) {
-        tmem_alloc(reinterpret_cast<uint32_t*>(&s.misc[0]), ncols);
-        tmem_relinquish();
+        if constexpr (kPair) {
+            tmem_alloc_pair(reinterpret_cast<uint32_t*>(&s.misc[0]), ncols);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(reinterpret_cast<uint32_t*>(&s.misc[0]), ncols);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (kPair) cluster_sync_all();  // the peer's barriers are initialised
     tc_fence_after();
     return static_cast<uint32_t>(s.misc[0]);
 }
 
+template <bool kPair = false>
 __device__ __forceinline__ void teardown(uint32_t tmem_base, int ncols) {
     tc_fence_before();
     __syncthreads();
+    if constexpr (kPair) cluster_sync_all();  // neither CTA leaves while the other may still signal it
     if ((threadIdx.x >> 5) == 1) {
         __syncwarp();
         tc_fence_after();
-        tmem_dealloc(tmem_base, ncols);
+        if constexpr (kPair) tmem_dealloc_pair(tmem_base, ncols);
+        else tmem_dealloc(tmem_base, ncols);
     }
 }
 
@@ -297,7 +423,14 @@ constexpr int lm_tmem_cols() {
 
 // ------------------------------------------------------------ LM-head kernel
 
-template <int NG>
+// kPair: two neighbouring vocabulary ranges of a node group as a CTA pair.
+// With 128-node groups the L2 -> SM bytes bound the launch (an SM takes in
+// about 64 bytes per clock): alone a CTA loads 16 KB of E and 32 KB of hi and
+// lo states per k-block, in a pair 16 KB of each.  Ranges, tiles and the order
+// of every sum are those of the single CTAs.  Measured on GB300, 256 nodes,
+// V = 151936, d = 4096 (µs per launch): single CTAs 450 (0.45 µs per k-block,
+// 107 GB/s into each SM), pairs with 4 stages 403, with 5 389.
+template <int NG, bool kPair>
 __global__ void __launch_bounds__(threads<NG>(), 1)
     lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmE, const __grid_constant__ CUtensorMap tmH,
                      const LmheadArgs a) {
@@ -305,7 +438,7 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
     pdl_trigger();
     const int stages = a.stages;
     constexpr int kNacc = lm_nacc<NG>();
-    Smem s = carve<NG>(smem_raw, stages, kNacc);
+    Smem s = carve<NG, kPair>(smem_raw, stages, kNacc);
     constexpr int kCap = lm_cand_cap<NG>();
     EpiSmem e;
     e.cap = kCap;
@@ -317,8 +450,9 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
     e.cnt = reinterpret_cast<int*>(e.mref + 4 * NG);
     e.more = e.cnt + NG;
 
-    const int g = blockIdx.x % a.G;
-    const int vr = blockIdx.x / a.G;
+    // (pairs: blocks 2 q and 2 q + 1 are ranges 2 r and 2 r + 1 of one group)
+    const int g = (kPair ? blockIdx.x / 2 : blockIdx.x) % a.G;
+    const int vr = kPair ? (blockIdx.x / 2 / a.G) * 2 + (blockIdx.x & 1) : blockIdx.x / a.G;
     const int t0 = static_cast<int>((static_cast<long long>(vr) * a.tiles) / a.nV);
     const int t1 = static_cast<int>((static_cast<long long>(vr + 1) * a.tiles) / a.nV);
     Work w;
@@ -331,16 +465,34 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
     w.tiled_kb = a.e_tiled ? w.kb1 : 0;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t tmem_base = setup<NG>(s, stages, lm_tmem_cols<NG>(), kNacc);
+    const uint32_t tmem_base = setup<NG, kPair>(s, stages, lm_tmem_cols<NG>(), kNacc);
     volatile int* abort = &s.misc[1];
+    // a pair walks as many tiles as its longer range: the shorter range's
+    // last accumulator (rows of the next range, or past V: zeros) is not read
+    const int own = w.ntiles;
+    if constexpr (kPair) {
+        const int o0 = static_cast<int>((static_cast<long long>(vr ^ 1) * a.tiles) / a.nV);
+        const int o1 = static_cast<int>((static_cast<long long>((vr ^ 1) + 1) * a.tiles) / a.nV);
+        w.ntiles = max(own, o1 - o0);
+    }
 
     if (warp == 0) {
-        if (lane == 0)
-            producer<NG>(&tmE, &tmH, w, a.bhalf, s.ring, stages, s.full, s.empty, abort, a.status, a.l2pf);
+        if (lane == 0) {
+            if constexpr (kPair)
+                producer_pair<NG>(&tmE, &tmH, w, blockIdx.x & 1, a.bhalf, s.ring, stages, s.full, s.empty, abort, a.status);
+            else
+                producer<NG>(&tmE, &tmH, w, a.bhalf, s.ring, stages, s.full, s.empty, abort, a.status, a.l2pf);
+        }
     } else if (warp == 1) {
-        if (lane == 0)
-            mma_issuer<NG>(w, s.ring, stages, s.full, s.empty, s.tfull, s.tempty, s.tdown, tmem_base,
-                           acc_stride<NG>(), abort, a.status, kNacc);
+        if constexpr (kPair) {
+            if (lane == 0 && (blockIdx.x & 1) == 0)
+                mma_issuer_pair<NG>(w, s.ring, stages, s.full, s.empty, s.tfull, s.tempty, s.tdown, tmem_base,
+                                    acc_stride<NG>(), abort, a.status, kNacc);
+        } else {
+            if (lane == 0)
+                mma_issuer<NG>(w, s.ring, stages, s.full, s.empty, s.tfull, s.tempty, s.tdown, tmem_base,
+                               acc_stride<NG>(), abort, a.status, kNacc);
+        }
     } else {
         // epilogue warp wi = warp - 2 reads TMEM lane quarter warp % 4 and
         // owns the 16-node chunks wi / 4 + 4 * ci (ci < kChunks) of the group
@@ -387,7 +539,17 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
                 }
             }
         };
-        for (int i = 0; i < w.ntiles; i++) {
+        // the accumulator has been read: the (leader's) next MMAs may overwrite it
+        auto release = [&](int acc) {
+            tc_fence_before();
+            if constexpr (kPair) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(mapa_u32(smem_u32(&s.tempty[acc]), 0));
+            } else {
+                mbar_arrive(&s.tempty[acc]);
+            }
+        };
+        for (int i = 0; i < own; i++) {
             const int acc = i % kNacc;
             const uint32_t aph = (i / kNacc) & 1;
             if (etid == 0) {
@@ -405,8 +567,7 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
                 // accumulator is released as soon as it has been read
                 float z[16];
                 load_z(acc, 0, v, valid, z);
-                tc_fence_before();
-                mbar_arrive(&s.tempty[acc]);
+                release(acc);
                 if (a.zout && valid) {
                     const int nb = g * NG + (wi >> 2) * 16;
 #pragma unroll
@@ -450,15 +611,14 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
                         }
                     }
                 }
-                tc_fence_before();
-                mbar_arrive(&s.tempty[acc]);
+                release(acc);
             }
         }
 #pragma unroll
         for (int ci = 0; ci < kChunks; ci++) epi_stash(e, NG, quarter, lane, ((wi >> 2) + 4 * ci) * 16, ssum[ci]);
         epi_finalize(e, NG, a.k, etid, kEpi, g * NG, a.N, vr, a.nV, a.part_ms, a.part_key);
     }
-    teardown(tmem_base, lm_tmem_cols<NG>());
+    teardown<kPair>(tmem_base, lm_tmem_cols<NG>());
 }
 
 // --------------------------------------------------------------- GEMM kernel
@@ -634,7 +794,12 @@ __global__ void __launch_bounds__(64) wait_probe_kernel(int* status, unsigned lo
 template <int NG>
 cudaError_t launch_lmhead_ng(const CUtensorMap* tmE, const CUtensorMap* tmH, const LmheadArgs& a, int smem,
                              cudaStream_t st) {
-    return launch_pdl(lmhead_tc_kernel<NG>, dim3(a.nV * a.G), dim3(threads<NG>()), smem, st, *tmE, *tmH, a);
+    if constexpr (NG == 128) {
+        if (a.pair)
+            return launch_pdl_cluster(lmhead_tc_kernel<NG, true>, dim3(a.nV * a.G), dim3(threads<NG>()), smem, st, 2,
+                                      *tmE, *tmH, a);
+    }
+    return launch_pdl(lmhead_tc_kernel<NG, false>, dim3(a.nV * a.G), dim3(threads<NG>()), smem, st, *tmE, *tmH, a);
 }
 template <int NG>
 cudaError_t launch_gemm_ng(const CUtensorMap* tmA, const CUtensorMap* tmB, const GemmArgs& a, int smem,
@@ -728,12 +893,18 @@ int gemm_tc_max_clusters(int NG, int smem, int cluster) {
 
 int lmhead_tc_ctas_per_sm(int NG, int smem) {
     switch (NG) {
-        case 16: return ctas_per_sm(reinterpret_cast<const void*>(lmhead_tc_kernel<16>), threads<16>(), smem);
-        case 32: return ctas_per_sm(reinterpret_cast<const void*>(lmhead_tc_kernel<32>), threads<32>(), smem);
-        case 64: return ctas_per_sm(reinterpret_cast<const void*>(lmhead_tc_kernel<64>), threads<64>(), smem);
-        default: return ctas_per_sm(reinterpret_cast<const void*>(lmhead_tc_kernel<128>), threads<128>(), smem);
+        case 16: return ctas_per_sm(reinterpret_cast<const void*>(lmhead_tc_kernel<16, false>), threads<16>(), smem);
+        case 32: return ctas_per_sm(reinterpret_cast<const void*>(lmhead_tc_kernel<32, false>), threads<32>(), smem);
+        case 64: return ctas_per_sm(reinterpret_cast<const void*>(lmhead_tc_kernel<64, false>), threads<64>(), smem);
+        default: return ctas_per_sm(reinterpret_cast<const void*>(lmhead_tc_kernel<128, false>), threads<128>(), smem);
     }
 }
+
+// Node groups from which two vocabulary ranges work as a CTA pair.  64-node
+// groups (16 + 16 KB per k-block alone) gain nothing from it: 136 µs per launch
+// either way at V = 151936, d = 2560, where HBM bounds them, and 3 x 11 nodes
+// at V = 50021, d = 1088 lost 4 %.
+constexpr int kLmheadPairNG = 128;
 
 bool plan_lmhead_tc(int N, int V, int d, int k, int num_sms, int smem_optin, int ctas_per_sm_pref, bool e_tiled,
                     LmheadPlan* out) {
@@ -742,7 +913,10 @@ bool plan_lmhead_tc(int N, int V, int d, int k, int num_sms, int smem_optin, int
     p.G = (N + p.NG - 1) / p.NG;
     const int tiles = (V + kTileM - 1) / kTileM;
     p.nV = std::max(1, std::min(num_sms / p.G, tiles));
-    const int sb = tc_stage_bytes(p.NG);
+    // CTA pairs: an even number of vocabulary ranges of at least one tile
+    const int nv1 = std::max(1, std::min(num_sms / p.G, tiles));
+    p.pair = p.NG >= kLmheadPairNG && nv1 % 2 == 0;
+    const int sb = p.pair ? kATileBytes + p.NG * 128 : tc_stage_bytes(p.NG);
     const int fixed = lmhead_tc_fixed_smem(p.NG, k, 16);
     auto stages_in = [&](int budget) { return std::min(16, (budget - fixed) / sb); };
     // Two CTAs per SM when both fit with >= 4 pipeline stages each: two
@@ -755,7 +929,7 @@ bool plan_lmhead_tc(int N, int V, int d, int k, int num_sms, int smem_optin, int
     const int st2 = stages_in(smem_optin / 2 - 2048);
     const int smem2 = lmhead_tc_fixed_smem(p.NG, k, st2) + st2 * sb;
     const bool want2 = ctas_per_sm_pref ? ctas_per_sm_pref == 2 : (e_tiled || d <= 3072);
-    if (want2 && st2 >= 4 && 2 * lmhead_tc_tmem_cols(p.NG) <= 512 && lmhead_tc_ctas_per_sm(p.NG, smem2) >= 2) {
+    if (!p.pair && want2 && st2 >= 4 && 2 * lmhead_tc_tmem_cols(p.NG) <= 512 && lmhead_tc_ctas_per_sm(p.NG, smem2) >= 2) {
         p.stages = st2;
         p.nV = std::max(1, std::min(2 * num_sms / p.G, tiles));
     } else {
@@ -773,10 +947,11 @@ cudaError_t tc_set_smem_limits(int max_dyn) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn); \
     if (e == cudaSuccess)                                                                              \
         e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    DART_SET(lmhead_tc_kernel<16>)
-    DART_SET(lmhead_tc_kernel<32>)
-    DART_SET(lmhead_tc_kernel<64>)
-    DART_SET(lmhead_tc_kernel<128>)
+    DART_SET((lmhead_tc_kernel<16, false>))
+    DART_SET((lmhead_tc_kernel<32, false>))
+    DART_SET((lmhead_tc_kernel<64, false>))
+    DART_SET((lmhead_tc_kernel<128, false>))
+    DART_SET((lmhead_tc_kernel<128, true>))
     DART_SET(gemm_tc_kernel<16>)
     DART_SET(gemm_tc_kernel<32>)
     DART_SET(gemm_tc_kernel<64>)
