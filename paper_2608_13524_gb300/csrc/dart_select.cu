@@ -495,35 +495,55 @@ __global__ void gather_silu_kernel(int Nc, int d, int S, int Np, const float* pa
 // One block per child: r = h[prow] + sum_s part[s], h_next = r / rms(r).
 // NT = 1024 threads when S partial tiles are summed (many loads in flight),
 // 256 for one summed tile (few registers, so blocks can become resident
-// beside the GEMM before it ends).
-template <int NT>
+// beside the GEMM before it ends).  kIt: float4 columns per thread, no more
+// than d needs, since the code is cold at every depth (one kernel for every d
+// was 20 to 55 KB).  Measured on GB300 against that one (µs per round, same
+// box): 3 x 11 nodes, d = 1088 565 -> 533, 64 nodes, d = 2560 2703 -> 2689,
+// 16 nodes, K = 64 466 -> 462; a cluster of four blocks per child was slower
+// where the LM-head follows (8 nodes 2071 -> 2096).
+template <int NT, int kIt>
 __global__ void __launch_bounds__(NT) residual_norm_kernel(int d, int S, int Nc, const float* part, const int* prow,
                                                            const float* h, float eps, float* h_next,
                                                            __nv_bfloat16* HL, int bhalf) {
     pdl_trigger();
     pdl_wait();
     __shared__ float red[32];
-    const int c = blockIdx.x;
+    const int c = blockIdx.x, lane = threadIdx.x & 31;
     const int pr = prow[c];
     const size_t total = static_cast<size_t>(Nc) * d;
-    constexpr int kMaxPer = 16384 / (4 * NT);  // d <= 16384
-    float4 r[kMaxPer];
-    float ss = 0.0f;
+    float4 r[kIt], q[kIt];
 #pragma unroll
-    for (int it = 0; it < kMaxPer; it++) {
+    for (int it = 0; it < kIt; it++) {
         const int j = (it * NT + threadIdx.x) * 4;
-        r[it] = make_float4(0.f, 0.f, 0.f, 0.f);
+        r[it] = q[it] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (j < d && pr >= 0) {
-            float4 v = *reinterpret_cast<const float4*>(h + static_cast<size_t>(pr) * d + j);
-            add_splits(v, part + static_cast<size_t>(c) * d + j, total, S);
-            r[it] = v;
-            ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+            r[it] = *reinterpret_cast<const float4*>(h + static_cast<size_t>(pr) * d + j);
+            q[it] = *reinterpret_cast<const float4*>(part + static_cast<size_t>(c) * d + j);
         }
     }
-    const float tot = block_sum_float(ss, red);
+    float ss = 0.0f;
+#pragma unroll
+    for (int it = 0; it < kIt; it++) {
+        const int j = (it * NT + threadIdx.x) * 4;
+        float4 v = r[it];
+        v.x += q[it].x;
+        v.y += q[it].y;
+        v.z += q[it].z;
+        v.w += q[it].w;
+        if (NT == 1024 && j < d && pr >= 0) add_splits(v, part + static_cast<size_t>(c) * d + j + total, total, S - 1);
+        r[it] = v;
+        ss = __fadd_rn(ss, fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.y, v.y, __fmul_rn(v.x, v.x)))));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(kFull, ss, o);
+    if (lane == 0) red[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    float tot = 0.0f;
+#pragma unroll 8
+    for (int i = 0; i < NT / 32; i++) tot += red[i];
     const float inv = 1.0f / sqrtf(tot / static_cast<float>(d) + eps);
 #pragma unroll
-    for (int it = 0; it < kMaxPer; it++) {
+    for (int it = 0; it < kIt; it++) {
         const int j = (it * NT + threadIdx.x) * 4;
         if (j < d) {
             const float4 v = make_float4(r[it].x * inv, r[it].y * inv, r[it].z * inv, r[it].w * inv);
@@ -633,11 +653,15 @@ bool debug_build() {
 
 cudaError_t launch_residual_norm(int Nc, int d, int S, const float* part, const int* prow, const float* h,
                                  float eps, float* h_next, __nv_bfloat16* HL, int bhalf, cudaStream_t st) {
-    if (S > 1)
-        return launch_pdl(residual_norm_kernel<1024>, dim3(Nc), dim3(1024), 0, st, d, S, Nc, part, prow, h, eps,
-                          h_next, HL, bhalf);
-    return launch_pdl(residual_norm_kernel<256>, dim3(Nc), dim3(256), 0, st, d, S, Nc, part, prow, h, eps, h_next,
-                      HL, bhalf);
+    const int NT = S > 1 ? 1024 : 256;
+    const int its = (d / 4 + NT - 1) / NT;  // (d <= 16384)
+    const auto fn = S > 1 ? (its <= 1   ? residual_norm_kernel<1024, 1>
+                             : its <= 2 ? residual_norm_kernel<1024, 2>
+                                        : residual_norm_kernel<1024, 4>)
+                          : (its <= 2   ? residual_norm_kernel<256, 2>
+                             : its <= 4 ? residual_norm_kernel<256, 4>
+                                        : residual_norm_kernel<256, 16>);
+    return launch_pdl(fn, dim3(Nc), dim3(NT), 0, st, d, S, Nc, part, prow, h, eps, h_next, HL, bhalf);
 }
 
 }  // namespace dart
