@@ -178,7 +178,7 @@ __device__ __forceinline__ void attn_drain(uint64_t* bar, uint32_t parity) {
 // A wait whose outcome is the same for every lane of the warp (the
 // tcgen05.ld / st that follow are warp-collective).
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-    const bool got = mbar_wait(bar, parity, abort);
+    const bool got = mbar_wait_inline(bar, parity, abort);
     return __all_sync(0xFFFFFFFFu, got);
 }
 
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                 const int key0 = (ctx ? j : j - a.nct) * kKeys;
                 if (do_k) {
                     const int st = i % kKStages;
-                    if (!mbar_wait(&k_empty[st], (static_cast<uint32_t>(i / kKStages) & 1u) ^ 1u, abort)) {
+                    if (!mbar_wait_inline(&k_empty[st], (static_cast<uint32_t>(i / kKStages) & 1u) ^ 1u, abort)) {
                         attn_timeout(a.status, abort);
                         break;
                     }
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     kdone++;
                 } else {
                     const int st = i % kVStages;
-                    if (!mbar_wait(&v_empty[st], (static_cast<uint32_t>(i / kVStages) & 1u) ^ 1u, abort)) {
+                    if (!mbar_wait_inline(&v_empty[st], (static_cast<uint32_t>(i / kVStages) & 1u) ^ 1u, abort)) {
                         attn_timeout(a.status, abort);
                         break;
                     }
@@ -425,12 +425,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (lane == 0 && nt > 0) {
             constexpr uint32_t idesc_s = idesc_bf16_f32(kRows, kKeys);
             constexpr uint32_t idesc_pv = idesc_bf16_f32(kRows, kDh) | (1u << 16);  // B (= V) MN-major
-            bool mok = mbar_wait(q_ready, 0, abort);
+            bool mok = mbar_wait_inline(q_ready, 0, abort);
             auto issue_s = [&](int i) -> bool {
                 const int st = i % kKStages;
                 // the S columns were last read by softmax(i - 1)
-                if (!mbar_wait(&k_full[st], static_cast<uint32_t>(i / kKStages) & 1u, abort) ||
-                    (i > 0 && !mbar_wait(s_empty, static_cast<uint32_t>(i - 1) & 1u, abort)))
+                if (!mbar_wait_inline(&k_full[st], static_cast<uint32_t>(i / kKStages) & 1u, abort) ||
+                    (i > 0 && !mbar_wait_inline(s_empty, static_cast<uint32_t>(i - 1) & 1u, abort)))
                     return false;
                 tc_fence_after();
                 const uint32_t k_addr = smem_u32(sK + st * kTileBytes);
@@ -452,8 +452,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     break;
                 }
                 const int st = i % kVStages;
-                if (!mbar_wait(p_full, static_cast<uint32_t>(i) & 1u, abort) ||
-                    !mbar_wait(&v_full[st], static_cast<uint32_t>(i / kVStages) & 1u, abort)) {
+                if (!mbar_wait_inline(p_full, static_cast<uint32_t>(i) & 1u, abort) ||
+                    !mbar_wait_inline(&v_full[st], static_cast<uint32_t>(i / kVStages) & 1u, abort)) {
                     mok = false;
                     break;
                 }

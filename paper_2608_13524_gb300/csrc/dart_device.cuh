@@ -131,8 +131,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // Waits for the phase with the given parity.  Gives up (returns false) when
 // *abort becomes nonzero or after limit_ns (kWaitLimitNs unless a test asks
 // for a shorter limit).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
-                                          unsigned long long limit_ns = kWaitLimitNs) {
+__device__ __forceinline__ bool mbar_wait_inline(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                                 unsigned long long limit_ns = kWaitLimitNs) {
     if (mbar_try_wait(bar, parity)) return true;
     const unsigned long long t0 = globaltimer_ns();
     for (;;) {
@@ -140,6 +140,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
         if (*abort) return false;
         if (globaltimer_ns() - t0 > limit_ns) return false;
     }
+}
+__device__ __noinline__ static bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                                  unsigned long long limit_ns) {
+    return mbar_wait_inline(bar, parity, abort, limit_ns);
+}
+// The same with the waiting loop out of line, for the kernels of a depth's
+// chain: each is cold when it starts, so its size counts.  (Where many warps
+// wait often the call costs more than it saves: tree attention, 8 sequences,
+// 191 -> 204 µs.)
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                          unsigned long long limit_ns = kWaitLimitNs) {
+    return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, abort, limit_ns);
 }
 
 // ----------------------------------------------------------------------- TMA
@@ -368,6 +380,7 @@ __device__ __forceinline__ uint64_t block_kth_largest(const uint64_t* keys, int 
     uint64_t prefix = 0, mask = 0;
     int remaining = kk;
     const int tid = threadIdx.x, nt = blockDim.x;
+#pragma unroll 1
     for (int shift = 56; shift >= 0; shift -= 8) {
         for (int i = tid; i < 256; i += nt) hist[i] = 0;
         __syncthreads();
@@ -604,6 +617,7 @@ __device__ __forceinline__ float warp_kth_largest(const float* y, int R, int kk,
     if (__any_sync(kFull, nan)) return __int_as_float(0x7FC00000);
     uint32_t prefix = 0, mask = 0;
     int need = kk;
+#pragma unroll 1
     for (int b = 31; b >= 0; b--) {
         const uint32_t bit = 1u << b, cand = prefix | bit, m2 = mask | bit;
         int cnt = 0;
@@ -628,7 +642,9 @@ __device__ __forceinline__ float warp_kth_largest(const float* y, int R, int kk,
 __device__ __forceinline__ void epi_init(const EpiSmem& e, int NG, int k, int etid, int nthr,
                                          uint64_t* gthr = nullptr, int n0 = 0, int N = 0,
                                          const float* seed_y = nullptr, int seed_R = 0, bool publish = false) {
+#pragma unroll 1
     for (int i = etid; i < NG * k; i += nthr) e.list[i] = 0ull;
+#pragma unroll 1
     for (int i = etid; i < NG; i += nthr) {
         e.cnt[i] = 0;
         if (!seed_y)
@@ -636,6 +652,7 @@ __device__ __forceinline__ void epi_init(const EpiSmem& e, int NG, int k, int et
     }
     if (seed_y) {
         const int lane = etid & 31;
+#pragma unroll 1
         for (int i = etid >> 5; i < NG; i += nthr >> 5) {
             uint64_t g = 0ull;
             if (n0 + i < N) {
@@ -652,6 +669,7 @@ __device__ __forceinline__ void epi_init(const EpiSmem& e, int NG, int k, int et
         }
     }
     if (etid < 2) e.more[etid] = 0;
+#pragma unroll 1
     for (int i = etid; i < 4 * NG; i += nthr) e.mref[i] = -INFINITY;
 }
 
@@ -764,6 +782,7 @@ __device__ __forceinline__ void warp_merge(uint64_t* L, const uint64_t* C, int c
         // few candidates: insert one at a time into the register-held list
         uint64_t a0 = lane < k ? L[lane] : 0ull;
         uint64_t a1 = lane + 32 < k ? L[lane + 32] : 0ull;
+#pragma unroll 1
         for (int i = 0; i < c; i++) {
             const uint64_t x = C[i];
             const int p = __popc(__ballot_sync(kFull, a0 > x)) + __popc(__ballot_sync(kFull, a1 > x));
@@ -780,6 +799,7 @@ __device__ __forceinline__ void warp_merge(uint64_t* L, const uint64_t* C, int c
         __syncwarp();
         return;
     }
+#pragma unroll 1
     for (int b = 0; b < c; b += 32) {
         const int nb = min(32, c - b);
         uint64_t x = lane < nb ? C[b + lane] : 0ull;
@@ -851,6 +871,7 @@ __device__ __forceinline__ void epi_merge(const EpiSmem& e, int NG, int k, int w
     if (reset_flag && etid == 0) *reset_flag = 0;  // every thread read it before this barrier
     uint64_t g = 0ull;
     if (gthr && etid < NG && n0 + etid < N) g = __ldcg(reinterpret_cast<const unsigned long long*>(gthr) + n0 + etid);
+#pragma unroll 1
     for (int nd = wi; nd < NG; nd += nthr / 32) {
         const int c = min(e.cnt[nd], e.cap);
         if (c == 0) continue;
@@ -889,13 +910,16 @@ __host__ __device__ __forceinline__ int part_stride(int nV, int k) { return (nV 
 __device__ __forceinline__ void epi_finalize(const EpiSmem& e, int NG, int k, int etid, int nthr, int n0, int N,
                                              int vr, int nV, float2* part_ms, uint64_t* part_key) {
     named_bar_sync(kEpiBarrier, nthr);
+#pragma unroll 1
     for (int c = etid; c < NG; c += nthr) {
         const int n = n0 + c;
         if (n >= N) continue;
         float2 a = e.stats[c];
+#pragma unroll 1
         for (int w = 1; w < 4; w++) a = lse_merge(a, e.stats[w * NG + c]);
         part_ms[static_cast<size_t>(n) * nV + vr] = a;
     }
+#pragma unroll 1
     for (int i = etid; i < NG * k; i += nthr) {
         const int c = i / k, j = i % k, n = n0 + c;
         if (n >= N) continue;

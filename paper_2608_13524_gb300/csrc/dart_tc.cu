@@ -111,6 +111,7 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmA, const CUtensorM
     // its first `pre` stages are requested before waiting on the previous
     // kernel; the B operand (node states) only after.
     const uint32_t pre = total < static_cast<uint32_t>(stages) ? total : static_cast<uint32_t>(stages);
+#pragma unroll 1
     for (uint32_t f = 0; f < pre; f++) {
         const int i = static_cast<int>(f) / kbs, kb = w.kb0 + static_cast<int>(f) % kbs;
         const bool lo = kb < w.lo_kb_end;
@@ -118,11 +119,13 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmA, const CUtensorM
         tma_load_2d(ring + f * Layout<NG>::kStage, tmA, &full[f], a_x(w, kb), a_y(w, i, kb), pol_a);
     }
     // and the next `l2pf` into L2, while the previous kernel still runs
+#pragma unroll 1
     for (uint32_t f = pre; f < pre + static_cast<uint32_t>(l2pf) && f < total; f++) {
         const int i = static_cast<int>(f) / kbs, kb = w.kb0 + static_cast<int>(f) % kbs;
         tma_prefetch_2d(tmA, a_x(w, kb), a_y(w, i, kb));
     }
     pdl_wait();
+#pragma unroll 1
     for (uint32_t f = 0; f < pre; f++) {
         const int kb = w.kb0 + static_cast<int>(f) % kbs;
         uint8_t* sH = ring + f * Layout<NG>::kStage + kATileBytes;
@@ -131,13 +134,18 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmA, const CUtensorM
     }
     uint32_t stage = pre % stages, phase = (pre / stages) & 1u, fills = pre;
     bool ok = true;
-    for (uint32_t f = pre; f < total; f++) {
+    int i = static_cast<int>(pre) / kbs, kb = w.kb0 + static_cast<int>(pre) % kbs;
+#pragma unroll 1
+    for (uint32_t f = pre; f < total; f++, kb++) {
+        if (kb == w.kb1) {
+            kb = w.kb0;
+            i++;
+        }
         if (!mbar_wait(&empty[stage], phase ^ 1u, abort)) {
             record_timeout(status, abort);
             ok = false;
             break;
         }
-        const int i = static_cast<int>(f) / kbs, kb = w.kb0 + static_cast<int>(f) % kbs;
         const bool lo = kb < w.lo_kb_end;
         uint8_t* sA = ring + stage * Layout<NG>::kStage;
         uint8_t* sH = sA + kATileBytes;
@@ -177,6 +185,7 @@ __device__ __forceinline__ void mma_issuer(const Work& w, uint8_t* ring, int sta
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * acc_stride;
+#pragma unroll 1
         for (int kb = w.kb0; kb < w.kb1; kb++) {
             if (!mbar_wait(&full[stage], phase, abort)) {
                 record_timeout(status, abort);
@@ -238,14 +247,17 @@ __device__ __forceinline__ void producer_pair(const CUtensorMap* tmA, const CUte
                          (w.kb0 + static_cast<int>(f) % kbs) * kBlockK, brow, pol_b);
     };
     // (as in `producer`: A does not depend on an earlier kernel, B does)
+#pragma unroll 1
     for (uint32_t f = 0; f < pre; f++) {
         if (rank == 0) mbar_arrive_expect_tx(&full[f], 2 * PairLayout<NG>::kStage);
         load_a(f, f);
     }
     pdl_wait();
+#pragma unroll 1
     for (uint32_t f = 0; f < pre; f++) load_b(f, f);
     uint32_t stage = pre % stages, phase = (pre / stages) & 1u, fills = pre;
     bool ok = true;
+#pragma unroll 1
     for (uint32_t f = pre; f < total; f++) {
         if (!mbar_wait(&empty[stage], phase ^ 1u, abort)) {
             record_timeout(status, abort);
@@ -294,6 +306,7 @@ __device__ __forceinline__ void mma_issuer_pair(const Work& w, uint8_t* ring, in
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * acc_stride;
+#pragma unroll 1
         for (int kb = w.kb0; kb < w.kb1; kb++) {
             if (!mbar_wait(&full[stage], phase, abort)) {
                 record_timeout(status, abort);
@@ -509,9 +522,16 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
         for (int ci = 0; ci < kChunks; ci++) {
             const int c0 = ((wi >> 2) + 4 * ci) * 16;
             ssum[ci] = 0.0f;
+            // bit j: node c0 + j exists; bit 16 + j: it starts a sequence (or the chunk)
             nodemask[ci] = 0;
-            for (int j = 0; j < 16; j++)
-                if (g * NG + c0 + j < a.N) nodemask[ci] |= 1u << j;
+            int left = 0;
+#pragma unroll 1
+            for (int j = 0; j < 16; j++) {
+                if (j == 0) left = a.P - (g * NG + c0) % a.P;
+                if (g * NG + c0 + j < a.N) nodemask[ci] |= (j == 0 || left == 0 ? 0x10001u : 1u) << j;
+                if (left == 0) left = a.P;
+                left--;
+            }
         }
         // scaled logits of this thread's row v for chunk ci from accumulator acc:
         // hi + lo products, drafter row added, 1/T applied
@@ -523,14 +543,13 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
             tmem_ld16_pair(tcol, tcol + NG, z, zl);
 #pragma unroll
             for (int j = 0; j < 16; j++) z[j] += zl[j];
-            int cur_seq = -1;
+            int seq = (g * NG + c0) / a.P - 1;
             float dl = 0.0f;
 #pragma unroll
             for (int j = 0; j < 16; j++) {
                 if ((nodemask[ci] >> j) & 1u) {
-                    const int seq = (g * NG + c0 + j) / a.P;
-                    if (seq != cur_seq) {
-                        cur_seq = seq;
+                    if ((nodemask[ci] >> (16 + j)) & 1u) {  // the first node of a sequence, or of the chunk
+                        seq++;
                         const long long off = a.dlog_row ? static_cast<long long>(__ldg(a.dlog_row + seq)) * a.V
                                                          : a.dlog_row_off;
                         dl = valid ? __ldg(a.dlog + seq * a.dlog_seq_stride + off + v) : 0.0f;
