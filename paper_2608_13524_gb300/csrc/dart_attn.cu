@@ -4,7 +4,7 @@
 // hands the pruned tree to that single forward pass).  Contract:
 // include/dart_verify.h.
 //
-// Two launches per call:
+// Launches of a call:
 //   attn_prep_kernel   the RoPE (cos, sin) table of every tree position and
 //                      the rotated tree keys (rotate-half RoPE in fp32,
 //                      rounded to bf16) in the workspace;
@@ -21,6 +21,9 @@
 //                      split over a thread-block cluster of up to 4 CTAs
 //                      that merge their partial (max, sum, O) over
 //                      distributed shared memory, in rank order;
+//   tree_attn2_kernel  the same for two query tiles per CTA, when there are
+//                      more query tiles than SMs (and tree_attn_kernel for
+//                      what its last wave would leave);
 // and dart_ancestor_mask's own kernel, one block per sequence.
 // tree_attn_kernel, 320 threads: warp 0 TMA producer (K ring 3 stages, V ring
 // 3 stages), warp 1 TMEM allocator + single-thread MMA issuer, warps 2-9 two
@@ -39,6 +42,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdint>
@@ -75,6 +79,8 @@ constexpr int kAttnSmem = kSmemUsed + 1024;  // + alignment slack of the 1024-by
 
 struct AttnArgs {
     int B, C, Hq, Hkv, G, qpt, nqt, splits, mw, nct;
+    int nunits;               // pairs of query tiles in all
+    int u0;                   // tree_attn_kernel: >= 0: blocks 2 i, 2 i + 1 are the query tiles of pair unit u0 + i
     float sl2;                // scale * log2(e)
     const float2* cs;         // [nseq][B][dh/2] RoPE (cos, sin) of the tree positions
     const int32_t* n_nodes;   // [nseq]
@@ -82,6 +88,16 @@ struct AttnArgs {
     float* out;               // [nseq][B][Hq][dh]
     int* status;
 };
+
+// Pair unit u (two neighbouring query tiles of a kv head): the pairs of the
+// last rows, which see the most tree keys, come first.
+__device__ __forceinline__ void pair_unit(const AttnArgs& a, int u, int* qp, int* kvh, int* s) {
+    const int nqp = (a.nqt + 1) / 2;
+    const int nsk = a.nunits / nqp;
+    *qp = nqp - 1 - u / nsk;
+    *kvh = (u % nsk) % a.Hkv;
+    *s = (u % nsk) / a.Hkv;
+}
 
 struct PrepArgs {
     int nseq, B, Hkv;
@@ -308,9 +324,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     // cluster rank is the key-range split
     const int split = a.splits > 1 ? static_cast<int>(cluster_ctarank()) : 0;
     const int blk = blockIdx.x / a.splits;
-    const int qt = blk % a.nqt;
-    const int kvh = (blk / a.nqt) % a.Hkv;
-    const int s = blk / (a.nqt * a.Hkv);
+    int qt = blk % a.nqt;
+    int kvh = (blk / a.nqt) % a.Hkv;
+    int s = blk / (a.nqt * a.Hkv);
+    if (a.u0 >= 0) {
+        pair_unit(a, a.u0 + blk / 2, &qt, &kvh, &s);
+        qt = 2 * qt + (blk & 1);
+        if (qt >= a.nqt) return;  // an odd number of query tiles: the last pair has one
+    }
     const int q0 = qt * a.qpt;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -482,6 +503,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             // first 64 and element t of the second 64 sit at the same
             // swizzled position of the two 16 KB halves; warpgroup wg
             // rotates chunks 4 wg .. 4 wg + 3
+            float4 f[16];  // (cos, sin) of this thread's 32 pairs, in flight while the queries load
+            const float4* cs = reinterpret_cast<const float4*>(a.cs + (static_cast<size_t>(s) * a.B + min(b, a.B - 1)) * (kDh / 2));
+#pragma unroll
+            for (int e = 0; e < 16; e++) f[e] = __ldg(cs + wg * 16 + e);
             if (!warp_wait(q_full, 0, abort)) {
                 attn_timeout(a.status, abort);
                 ok = false;
@@ -491,7 +516,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             // columns kQCol + t / 2 and kQCol + 32 + t / 2 (zeros past row B)
             uint32_t q1[16], q2[16];
             if (ok && b < a.B) {
-                const float4* cs = reinterpret_cast<const float4*>(a.cs + (static_cast<size_t>(s) * a.B + b) * (kDh / 2));
 #pragma unroll
                 for (int cc = 0; cc < 4; cc++) {
                     const int c = wg * 4 + cc;
@@ -502,13 +526,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     const uint32_t* u2 = reinterpret_cast<const uint32_t*>(&x2);
 #pragma unroll
                     for (int e = 0; e < 4; e++) {
-                        const float4 f = __ldg(cs + c * 4 + e);  // (cos, sin) of pairs 8c+2e, 8c+2e+1
+                        const float4 cw = f[cc * 4 + e];  // pairs 8c+2e, 8c+2e+1
                         const __nv_bfloat162 h1 = *reinterpret_cast<const __nv_bfloat162*>(&u1[e]);
                         const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&u2[e]);
                         const float a0 = __low2float(h1), a1 = __high2float(h1);
                         const float b0 = __low2float(h2), b1 = __high2float(h2);
-                        q1[cc * 4 + e] = pack_bf16(a0 * f.x - b0 * f.y, a1 * f.z - b1 * f.w);
-                        q2[cc * 4 + e] = pack_bf16(b0 * f.x + a0 * f.y, b1 * f.z + a1 * f.w);
+                        q1[cc * 4 + e] = pack_bf16(a0 * cw.x - b0 * cw.y, a1 * cw.z - b1 * cw.w);
+                        q2[cc * 4 + e] = pack_bf16(b0 * cw.x + a0 * cw.y, b1 * cw.z + a1 * cw.w);
                     }
                 }
             } else {
@@ -751,6 +775,425 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     }
 }
 
+// ------------------------------------------------------------ attention, two query tiles
+//
+// The kernel for more (sequence, kv head, query tile) blocks than SMs: a CTA
+// owns two neighbouring query tiles of a kv head, two softmax warpgroups each
+// (thread = query row = TMEM lane, 64 keys of a tile), so that one tile's
+// MMAs run during the other's softmax and every K/V tile is read once for
+// both.  Order of the issuing thread: S0(0), S1(0); then per key tile i
+// PV0(i), S0(i+1), PV1(i), S1(i+1).  The tensor pipe queues hardly anything,
+// so all that this thread does besides (a wait takes it 100 cycles even when
+// it is satisfied) leaves the pipe idle: two helper warps wait for the K and V
+// tiles and free their slots, and it waits and commits once per tile.  P_t overwrites the first 64 columns of
+// S_t (the MMAs are in order: PV_t(i) has read it before S_t(i+1) is
+// written), and a tile's S being complete implies that its previous PV is, so
+// O_t may be rescaled without another wait.  TMEM: S0 [0,128), S1 [128,256),
+// O0 [256,384), O1 [384,512); the rotated queries stay in shared memory.
+// Every row's maxima, probabilities and sums are those of tree_attn_kernel,
+// tile by tile, so both give the same output.
+// Measured on GB300, 8 x 512 rows, 32 / 8 heads, 2048 context keys: 190 µs per
+// call with one query tile per CTA, 163 with pairs.  A key tile takes a pair
+// 4000 cycles (2 x 1900 alone) of which the issuing thread spends 3250 on 32
+// MMAs: beside the softmax's TMEM and shared-memory traffic one costs 100
+// cycles instead of 65.  Tried: an issuing thread per query tile (223 µs),
+// the waits and the freeing of slots in the issuing thread (198), one
+// warpgroup per query tile (196).
+constexpr int kK2Stages = 3, kV2Stages = 2;
+constexpr int kNum2Bars = 1 + 2 * kK2Stages + 2 * kV2Stages + 2 * 4 + 1;
+constexpr int kSmem2Used =
+    kTileBytes * (2 + kK2Stages + kV2Stages) + kNum2Bars * 8 + 4 * 4 + 2 * 2 * 128 * 4 + 2 * 8 * 4;  // ... exchange
+constexpr int kFirstSoft2 = 4;                       // first softmax warp
+constexpr int kAttn2Threads = kFirstSoft2 * 32 + 512;
+constexpr int kAttn2Smem = kSmem2Used;  // (the base is declared with the swizzle atoms' 1024-byte alignment)
+
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, const void* src, int x, int y, int z, int w) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(smem_u32(src)), "r"(x), "r"(y), "r"(z), "r"(w)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(kAttn2Threads, 1)
+    tree_attn2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKc,
+                      const __grid_constant__ CUtensorMap tmVc, const __grid_constant__ CUtensorMap tmKt,
+                      const __grid_constant__ CUtensorMap tmVt,
+                      const __grid_constant__ CUtensorMap tmO, const AttnArgs a) {
+    extern __shared__ __align__(1024) uint8_t attn2_smem[];
+    pdl_trigger();
+    uint8_t* sQ = attn2_smem;                         // [2] query tiles
+    uint8_t* sK = sQ + 2 * kTileBytes;
+    uint8_t* sV = sK + kK2Stages * kTileBytes;
+    uint64_t* q_full = reinterpret_cast<uint64_t*>(sV + kV2Stages * kTileBytes);
+    uint64_t* k_full = q_full + 1;
+    uint64_t* k_empty = k_full + kK2Stages;
+    uint64_t* v_full = k_empty + kK2Stages;
+    uint64_t* v_empty = v_full + kV2Stages;
+    uint64_t* q_ready = v_empty + kV2Stages;          // [2] the tile's queries are rotated
+    uint64_t* s_full = q_ready + 2;                   // [2]
+    uint64_t* p_full = s_full + 2;                    // [2]
+    uint64_t* o_full = p_full + 2;                    // [2] the last PV of the tile is done
+    uint64_t* tdown = o_full + 2;
+    int* misc = reinterpret_cast<int*>(q_full + kNum2Bars);  // [0] TMEM base, [1] abort
+    volatile int* abort = &misc[1];
+    float* xch = reinterpret_cast<float*>(misc + 4);  // [2 tiles][2 warpgroups][128] row max / sum
+    int* xok = reinterpret_cast<int*>(xch + 2 * 2 * kRows);  // [2][2][4] per-warp "no wait failed"
+
+    int qp, kvh, s;
+    pair_unit(a, blockIdx.x, &qp, &kvh, &s);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        mbar_init(q_full, 1);
+        for (int i = 0; i < kK2Stages; i++) {
+            mbar_init(&k_full[i], 1);
+            mbar_init(&k_empty[i], 1);
+        }
+        for (int i = 0; i < kV2Stages; i++) {
+            mbar_init(&v_full[i], 1);
+            mbar_init(&v_empty[i], 1);
+        }
+        for (int t = 0; t < 2; t++) {
+            mbar_init(&q_ready[t], 8);
+            mbar_init(&s_full[t], 1);
+            mbar_init(&p_full[t], 9);
+            mbar_init(&o_full[t], 1);
+        }
+        mbar_init(tdown, 1);
+        misc[1] = 0;
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(reinterpret_cast<uint32_t*>(&misc[0]), kTmemCols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = static_cast<uint32_t>(misc[0]);
+    pdl_wait();
+
+    const int nn = min(max(__ldg(a.n_nodes + s), 0), a.B);
+    // key tiles of each query tile: 0 if none of its rows is a node
+    int nt[2];
+#pragma unroll
+    for (int t = 0; t < 2; t++) {
+        const int q0 = (2 * qp + t) * a.qpt, qlast = min(q0 + a.qpt, nn) - 1;
+        nt[t] = qlast >= q0 ? a.nct + qlast / kKeys + 1 : 0;
+    }
+    const int ntm = max(nt[0], nt[1]);
+
+    if (warp == 0) {
+        if (lane == 0 && ntm > 0) {
+            const uint64_t pol_q = l2_policy_evict_first();
+            const uint64_t pol_kv = l2_policy_evict_last();  // re-read by the other query tiles
+            mbar_arrive_expect_tx(q_full, 2 * kTileBytes);
+            for (int t = 0; t < 2; t++)
+                for (int hf = 0; hf < 2; hf++)  // (rows past B are filled with zeros)
+                    tma_load_4d(sQ + t * kTileBytes + hf * kHalf, &tmQ, q_full, hf * 64, kvh * a.G, (2 * qp + t) * a.qpt, s,
+                                pol_q);
+            int kdone = 0, vdone = 0;
+            while ((kdone < ntm || vdone < ntm) && !*abort) {
+                const bool do_k = kdone < ntm && kdone < vdone + 2;  // K one tile ahead of V
+                const int i = do_k ? kdone : vdone;
+                const bool ctx = i < a.nct;
+                const int key0 = (ctx ? i : i - a.nct) * kKeys;
+                const int ns = do_k ? kK2Stages : kV2Stages;
+                uint64_t* full = (do_k ? k_full : v_full) + i % ns;
+                uint64_t* empty = (do_k ? k_empty : v_empty) + i % ns;
+                if (!mbar_wait_inline(empty, (static_cast<uint32_t>(i / ns) & 1u) ^ 1u, abort)) {
+                    attn_timeout(a.status, abort);
+                    break;
+                }
+                uint8_t* dst = (do_k ? sK : sV) + (i % ns) * kTileBytes;
+                const CUtensorMap* tm = do_k ? (ctx ? &tmKc : &tmKt) : (ctx ? &tmVc : &tmVt);
+                mbar_arrive_expect_tx(full, kTileBytes);
+                tma_load_4d(dst, tm, full, 0, kvh, key0, s, pol_kv);
+                tma_load_4d(dst + kHalf, tm, full, 64, kvh, key0, s, pol_kv);
+                (do_k ? kdone : vdone)++;
+            }
+            if (*abort) {
+                // copies still in flight must land before the CTA exits
+                attn_drain(q_full, 0);
+                for (int i = max(kdone - kK2Stages, 0); i < kdone; i++)
+                    attn_drain(&k_full[i % kK2Stages], static_cast<uint32_t>(i / kK2Stages) & 1u);
+                for (int i = max(vdone - kV2Stages, 0); i < vdone; i++)
+                    attn_drain(&v_full[i % kV2Stages], static_cast<uint32_t>(i / kV2Stages) & 1u);
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0 && ntm > 0) {
+            constexpr uint32_t idesc_s = idesc_bf16_f32(kRows, kKeys);
+            constexpr uint32_t idesc_pv = idesc_bf16_f32(kRows, kDh) | (1u << 16);  // B (= V) MN-major
+            constexpr int kTile16 = kTileBytes >> 4, kHalf16 = kHalf >> 4;  // (descriptors address units of 16 bytes)
+            const uint64_t q_desc = sdesc_sw128(smem_u32(sQ)), k_desc = sdesc_sw128(smem_u32(sK));
+            const uint64_t v_desc = sdesc_sw128_mn(smem_u32(sV), kHalf);
+            const int nt0 = nt[0], nt1 = nt[1];
+            auto issue_s = [&](int t, int ks) {
+                const uint64_t qd = q_desc + t * kTile16, kd = k_desc + ks * kTile16;
+#pragma unroll
+                for (int kk = 0; kk < kDh / 16; kk++) {
+                    const int o = (kk >> 2) * kHalf16 + (kk & 3) * 2;
+                    tc_mma_bf16(tmem + t * 128, qd + o, kd + o, idesc_s, kk > 0 ? 1u : 0u);
+                }
+                tc_commit(&s_full[t]);
+            };
+            auto step = [&](int t, int i, int my_nt, int ks, int vs) -> bool {
+                // (P(i) written, V(i) and K(i + 1) loaded)
+                if (!mbar_wait_inline(&p_full[t], static_cast<uint32_t>(i) & 1u, abort)) return false;
+                tc_fence_after();
+                const uint64_t vd = v_desc + vs * kTile16;
+#pragma unroll
+                for (int kk = 0; kk < kKeys / 16; kk++)  // 16 keys = 8 columns of bf16 pairs
+                    tc_mma_bf16_ts(tmem + 256 + t * 128, tmem + t * 128 + kk * 8, vd + kk * (2048 >> 4), idesc_pv,
+                                   (i > 0 || kk > 0) ? 1u : 0u);
+                if (i + 1 < my_nt) issue_s(t, ks);
+                else tc_commit(&o_full[t]);
+                return true;
+            };
+            bool ok = mbar_wait_inline(&k_full[0], 0, abort);
+            if (ok && nt0 > 0) {
+                ok = mbar_wait_inline(&q_ready[0], 0, abort);
+                tc_fence_after();
+                if (ok) issue_s(0, 0);
+            }
+            if (ok && nt1 > 0) {
+                ok = mbar_wait_inline(&q_ready[1], 0, abort);
+                tc_fence_after();
+                if (ok) issue_s(1, 0);
+            }
+            int ks = 0, vs = 0;
+#pragma unroll 1
+            for (int i = 0; i < ntm && ok; i++) {
+                ks = ks + 1 == kK2Stages ? 0 : ks + 1;  // slot of K tile i + 1
+                if (i < nt0) ok = step(0, i, nt0, ks, vs);
+                if (ok && i < nt1) ok = step(1, i, nt1, ks, vs);
+                vs = vs + 1 == kV2Stages ? 0 : vs + 1;
+            }
+            if (!ok) {
+                attn_timeout(a.status, abort);
+                tc_commit(tdown);
+                attn_drain(tdown, 0);
+            }
+        }
+    } else if (warp < kFirstSoft2) {
+        // warp 2 + t waits, for the issuing thread, for the V and K tiles of
+        // the next step of query tile t (a ninth arrival at p_full), and for
+        // the last tile in issue order it frees the slots: S(i) complete
+        // means that K(i) and V(i - 1) have been read
+        const int t = warp - 2;
+        const bool frees = t == (nt[1] > 0 ? 1 : 0);  // (nt[0] <= nt[1] unless nt[1] = 0)
+        if (lane == 0) {
+            bool ok = true;
+#pragma unroll 1
+            for (int i = 0; i < nt[t] && ok; i++) {
+                if (frees) {
+                    ok = mbar_wait_inline(&s_full[t], static_cast<uint32_t>(i) & 1u, abort);
+                    if (!ok) break;
+                    mbar_arrive(&k_empty[i % kK2Stages]);
+                    if (i > 0) mbar_arrive(&v_empty[(i - 1) % kV2Stages]);
+                }
+                ok = mbar_wait_inline(&v_full[i % kV2Stages], static_cast<uint32_t>(i / kV2Stages) & 1u, abort) &&
+                     (i + 1 >= ntm || mbar_wait_inline(&k_full[(i + 1) % kK2Stages],
+                                                       static_cast<uint32_t>((i + 1) / kK2Stages) & 1u, abort));
+                if (!ok) break;
+                mbar_arrive(&p_full[t]);
+                ok = mbar_wait_inline(&p_full[t], static_cast<uint32_t>(i) & 1u, abort);
+            }
+            if (!ok) attn_timeout(a.status, abort);
+        }
+    } else {
+        // two warpgroups per query tile: warpgroup (t, wg) takes key and O
+        // columns [64 wg, 64 wg + 64) of the rows of tile 2 qp + t; the two
+        // warps of a lane quarter exchange their row maxima
+        const int sw = warp - kFirstSoft2;
+        const int t = sw >> 3, wg = (sw >> 2) & 1, qd = warp & 3, r = qd * 32 + lane;
+        const int cb = wg * 64, pair_bar = kPairBarrier0 + t * 4 + qd;
+        const int my_nt = t ? nt[1] : nt[0];
+        const int b = (2 * qp + t) * a.qpt + r / a.G, g = r % a.G;
+        const bool row_ok = b < nn;
+        const uint32_t tS = tmem + t * 128 + (static_cast<uint32_t>(qd * 32) << 16), tO = tS + 256 + cb;
+        float* xt = xch + t * 2 * kRows;       // [2 warpgroups][128]
+        int* xk = xok + t * 8 + qd;            // [2 warpgroups][4]
+        float m_run = -INFINITY, l = 0.0f;
+        bool ok = true;
+        if (my_nt > 0) {
+            // rotate this row's chunks 4 wg .. 4 wg + 3 in place (element e of
+            // the first 64 and of the second 64 sit at the same swizzled
+            // position of the two 16 KB halves)
+            float4 f[16];  // (cos, sin) of this thread's 32 pairs, in flight while the queries load
+            const float4* cs = reinterpret_cast<const float4*>(a.cs + (static_cast<size_t>(s) * a.B + min(b, a.B - 1)) * (kDh / 2));
+#pragma unroll
+            for (int e = 0; e < 16; e++) f[e] = __ldg(cs + wg * 16 + e);
+            ok = warp_wait(q_full, 0, abort);
+            if (ok && b < a.B) {
+#pragma unroll
+                for (int cc = 0; cc < 4; cc++) {
+                    const int c = wg * 4 + cc;
+                    uint8_t* p1 = sQ + t * kTileBytes + r * 128 + ((static_cast<uint32_t>(c) ^ (r & 7)) << 4);
+                    uint4 x1 = *reinterpret_cast<const uint4*>(p1);
+                    uint4 x2 = *reinterpret_cast<const uint4*>(p1 + kHalf);
+                    uint32_t* u1 = reinterpret_cast<uint32_t*>(&x1);
+                    uint32_t* u2 = reinterpret_cast<uint32_t*>(&x2);
+#pragma unroll
+                    for (int e = 0; e < 4; e++) {
+                        const float4 w = f[cc * 4 + e];  // pairs 8c+2e, 8c+2e+1
+                        const __nv_bfloat162 h1 = *reinterpret_cast<const __nv_bfloat162*>(&u1[e]);
+                        const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&u2[e]);
+                        const float a0 = __low2float(h1), a1 = __high2float(h1);
+                        const float b0 = __low2float(h2), b1 = __high2float(h2);
+                        u1[e] = pack_bf16(a0 * w.x - b0 * w.y, a1 * w.z - b1 * w.w);
+                        u2[e] = pack_bf16(b0 * w.x + a0 * w.y, b1 * w.z + a1 * w.w);
+                    }
+                    *reinterpret_cast<uint4*>(p1) = x1;
+                    *reinterpret_cast<uint4*>(p1 + kHalf) = x2;
+                }
+            }
+            if (!ok) attn_timeout(a.status, abort);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the MMAs read it
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&q_ready[t]);
+        }
+#pragma unroll 1
+        for (int i = 0; i < my_nt; i++) {
+            uint64_t w = 0ull;  // visible keys of this row among this warpgroup's 64
+            if (row_ok) {
+                int kvalid;
+                if (i < a.nct) {
+                    kvalid = min(kKeys, a.C - i * kKeys) - cb;
+                    w = ~0ull;
+                } else {
+                    const int wd = 2 * (i - a.nct) + wg;
+                    kvalid = nn - wd * 64;
+                    if (wd < a.mw) w = __ldg(a.mask + (static_cast<size_t>(s) * a.B + b) * a.mw + wd);
+                }
+                if (kvalid <= 0)
+                    w = 0ull;
+                else if (kvalid < 64)
+                    w &= (1ull << kvalid) - 1ull;
+            }
+            const bool full = __all_sync(0xFFFFFFFFu, w == ~0ull);  // the whole warp sees all 64 keys
+            // Both warps of a lane quarter reach the pair barrier of every
+            // iteration and leave the loop together: a failed wait is
+            // exchanged with the row max.
+            if (ok && !warp_wait(&s_full[t], static_cast<uint32_t>(i) & 1u, abort)) {
+                attn_timeout(a.status, abort);
+                ok = false;
+            }
+            float sv[64];
+            float mx = -INFINITY;
+            if (ok) {
+                tc_fence_after();
+                tmem_ld64(tS + cb, sv);
+                if (full) {
+#pragma unroll
+                    for (int c = 0; c < 64; c += 2) mx = fmaxf(mx, fmaxf(sv[c], sv[c + 1]));
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 64; c++) {
+                        if (!((w >> c) & 1ull)) sv[c] = -INFINITY;
+                        mx = fmaxf(mx, sv[c]);
+                    }
+                }
+            }
+            // (S(i) complete: the other warp has arrived at p_full(i - 1),
+            // after it read the previous exchange)
+            xt[wg * kRows + r] = mx;
+            if (lane == 0) xk[wg * 4] = ok ? 1 : 0;
+            named_bar_sync(pair_bar, 64);  // also: both halves of S are in registers (P overwrites them)
+            mx = fmaxf(mx, xt[(1 - wg) * kRows + r]);
+            ok = ok && xk[(1 - wg) * 4] != 0;
+            if (!ok) break;
+            const float mx2 = mx * a.sl2;
+            const bool resc = mx2 > m_run + kRescaleSlack;
+            const float m_new = resc ? mx2 : m_run;
+            const float alpha = resc ? ex2(m_run - m_new) : 1.0f;
+            if (i > 0 && __any_sync(0xFFFFFFFFu, resc)) {
+                // (S(i) complete: PV(i - 1) is too)
+#pragma unroll 1
+                for (int c0 = 0; c0 < 64; c0 += 16) {
+                    float o[16];
+                    tmem_ld16(tO + c0, o);
+#pragma unroll
+                    for (int e = 0; e < 16; e++) o[e] *= alpha;
+                    tmem_st16(tO + c0, o);
+                }
+            }
+            l *= alpha;
+            m_run = m_new;
+            const float nm = m_run == -INFINITY ? 0.0f : -m_run;
+            float lsum = 0.0f;
+#pragma unroll
+            for (int hf = 0; hf < 2; hf++) {
+                uint32_t pk[16];
+#pragma unroll
+                for (int c = 0; c < 32; c += 2) {
+                    const float p0 = ex2(fmaf(sv[hf * 32 + c], a.sl2, nm));
+                    const float p1 = ex2(fmaf(sv[hf * 32 + c + 1], a.sl2, nm));
+                    lsum += p0 + p1;
+                    pk[c >> 1] = pack_bf16(p0, p1);
+                }
+                tmem_st16u(tS + wg * 32 + hf * 16, pk);
+            }
+            tmem_wait_st();
+            l += lsum;
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&p_full[t]);
+        }
+        // both tiles' MMAs done: queries and K/V are no longer read
+#pragma unroll 1
+        for (int u = 0; u < 2; u++) {
+            if (ok && nt[u] > 0 && !warp_wait(&o_full[u], 0, abort)) {
+                attn_timeout(a.status, abort);
+                ok = false;
+            }
+        }
+        tc_fence_after();
+        // the row sum is split over the two warpgroups
+        xt[wg * kRows + r] = l;
+        named_bar_sync(pair_bar, 64);
+        l += xt[(1 - wg) * kRows + r];
+        const float inv = (row_ok && l > 0.0f) ? 1.0f / l : 0.0f;
+        // O / l into shared memory (tile 0 over the queries, tile 1 over K) in
+        // the swizzled layout of the store, which clips rows past B: four
+        // boxes of 32 columns per tile, two per warpgroup.  (Rows lie 512 bytes
+        // apart: stored by their own threads they took 4 µs of a CTA's 50.)
+        uint8_t* ob = t ? sK : sQ;
+#pragma unroll 1
+        for (int c0 = 0; c0 < 64; c0 += 16) {
+            float o[16];
+            if (my_nt > 0) {
+                tmem_ld16(tO + c0, o);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 16; e++) o[e] = 0.0f;
+            }
+            uint8_t* row = ob + (cb + c0) / 32 * kHalf + r * 128;
+            const int ch = (c0 & 16) / 4;  // first 16-byte chunk of the row
+#pragma unroll
+            for (int e = 0; e < 4; e++)
+                *reinterpret_cast<float4*>(row + (((ch + e) ^ (r & 7)) << 4)) =
+                    make_float4(o[4 * e] * inv, o[4 * e + 1] * inv, o[4 * e + 2] * inv, o[4 * e + 3] * inv);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        named_bar_sync(kPairBarrier0 + 8 + t * 2 + wg, 128);
+        const int q0 = (2 * qp + t) * a.qpt;
+        if ((sw & 3) == 0 && lane == 0 && q0 < a.B) {
+            for (int q = 2 * wg; q < 2 * wg + 2; q++) tma_store_4d(&tmO, ob + q * kHalf, q * 32, kvh * a.G, q0, s);
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc(tmem, kTmemCols);
+    }
+}
+
 // ------------------------------------------------------------ ancestor mask
 
 constexpr int kMaskThreads = 1024;
@@ -876,6 +1319,21 @@ bool encode_q(CUtensorMap* m, const void* base, int nseq, int B, int Hq, int G, 
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The output [nseq][B][Hq][dh] fp32 with a (32, G heads, qpt rows, 1) box.
+bool encode_out(CUtensorMap* m, void* base, int nseq, int B, int Hq, int G, int qpt) {
+    EncodeTiledFn fn = tensor_map_encoder();
+    if (!fn) return false;
+    cuuint64_t dims[4] = {static_cast<cuuint64_t>(kDh), static_cast<cuuint64_t>(Hq), static_cast<cuuint64_t>(B),
+                          static_cast<cuuint64_t>(nseq)};
+    cuuint64_t strides[3] = {static_cast<cuuint64_t>(kDh) * 4, static_cast<cuuint64_t>(Hq) * kDh * 4,
+                             static_cast<cuuint64_t>(B) * Hq * kDh * 4};
+    cuuint32_t box[4] = {32, static_cast<cuuint32_t>(G), static_cast<cuuint32_t>(qpt), 1};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+           CUDA_SUCCESS;
+}
+
 // [nseq][len][Hkv][dh] bf16 with a (64, 1, 128 keys, 1) box.
 bool encode_kv(CUtensorMap* m, const void* base, int nseq, int len, int Hkv) {
     EncodeTiledFn fn = tensor_map_encoder();
@@ -900,7 +1358,8 @@ bool attn_attr_set(int dev) {
     const uint64_t bit = dev < 64 ? (1ull << dev) : 0ull;
     if (bit && (done.load() & bit)) return true;
     if (cudaFuncSetAttribute(tree_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem) !=
-        cudaSuccess)
+            cudaSuccess ||
+        cudaFuncSetAttribute(tree_attn2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttn2Smem) != cudaSuccess)
         return false;
     done.fetch_or(bit);
     return true;
@@ -928,7 +1387,7 @@ int enqueue_tree_attention(const dart_attn_config* cfg, const void* q, const voi
     int dev = 0;
     DevInfo di;
     if (cudaGetDevice(&dev) != cudaSuccess || !dev_info(dev, &di)) return DART_ERR_CUDA;
-    if (di.major != 10 || di.minor != 3 || di.optin < kAttnSmem) return DART_ERR_UNSUPPORTED;
+    if (di.major != 10 || di.minor != 3 || di.optin < std::max(kAttnSmem, kAttn2Smem)) return DART_ERR_UNSUPPORTED;
     const int nsm = di.nsm > 0 ? di.nsm : 148;
     const Plan p = make_plan(cfg, nsm);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -936,7 +1395,9 @@ int enqueue_tree_attention(const dart_attn_config* cfg, const void* q, const voi
     __nv_bfloat16* kr = reinterpret_cast<__nv_bfloat16*>(ws + wl.off_kr);
     float2* cs = reinterpret_cast<float2*>(ws + wl.off_cs);
 
-    CUtensorMap tmQ, tmKc, tmVc, tmKt, tmVt;
+    const bool two = p.splits == 1 && p.blocks > nsm;  // two query tiles per CTA (tree_attn2_kernel)
+    CUtensorMap tmQ, tmKc, tmVc, tmKt, tmVt, tmO;
+    if (two && !encode_out(&tmO, out, c.nseq, c.B, c.Hq, p.G, p.qpt)) return DART_ERR_CUDA;
     if (!encode_q(&tmQ, q, c.nseq, c.B, c.Hq, p.G, p.qpt)) return DART_ERR_CUDA;
     if (!encode_kv(&tmKt, kr, c.nseq, c.B, c.Hkv) || !encode_kv(&tmVt, v_tree, c.nseq, c.B, c.Hkv))
         return DART_ERR_CUDA;
@@ -972,6 +1433,8 @@ int enqueue_tree_attention(const dart_attn_config* cfg, const void* q, const voi
     aa.splits = p.splits;
     aa.mw = p.mw;
     aa.nct = p.nct;
+    aa.nunits = c.nseq * c.Hkv * ((p.nqt + 1) / 2);
+    aa.u0 = -1;
     aa.sl2 = static_cast<float>(static_cast<double>(c.scale) * 1.4426950408889634);
     aa.cs = cs;
     aa.n_nodes = n_nodes;
@@ -985,11 +1448,28 @@ int enqueue_tree_attention(const dart_attn_config* cfg, const void* q, const voi
     if (ev && cudaEventRecord(ev[0], st) != cudaSuccess) return DART_ERR_CUDA;
     if (launch_pdl(attn_prep_kernel, dim3(prep_blocks), dim3(256), 0, st, ra) != cudaSuccess) return DART_ERR_CUDA;
     if (ev && cudaEventRecord(ev[1], st) != cudaSuccess) return DART_ERR_CUDA;
-    const cudaError_t le =
-        p.splits > 1 ? launch_pdl_cluster(tree_attn_kernel, dim3(p.blocks * p.splits), dim3(kAttnThreads), kAttnSmem,
-                                          st, p.splits, tmQ, tmKc, tmVc, tmKt, tmVt, aa)
-                     : launch_pdl(tree_attn_kernel, dim3(p.blocks), dim3(kAttnThreads), kAttnSmem, st, tmQ, tmKc,
-                                  tmVc, tmKt, tmVt, aa);
+    cudaError_t le;
+    if (two) {
+        // Whole waves of pairs; a last wave that would leave half of the SMs
+        // idle goes to tree_attn_kernel, one query tile per CTA.  Measured on
+        // GB300, 512 pairs on 152 SMs (8 x 512 rows, 2048 context keys): four
+        // waves of pairs 175 µs, three and 112 single tiles 163.
+        const int rem = aa.nunits % nsm;
+        const int single = aa.nunits > nsm && 2 * rem <= nsm ? rem : 0;
+        le = launch_pdl(tree_attn2_kernel, dim3(aa.nunits - single), dim3(kAttn2Threads), kAttn2Smem, st, tmQ, tmKc, tmVc,
+                        tmKt, tmVt, tmO, aa);
+        if (le == cudaSuccess && single > 0) {
+            aa.u0 = aa.nunits - single;
+            le = launch_pdl(tree_attn_kernel, dim3(2 * single), dim3(kAttnThreads), kAttnSmem, st, tmQ, tmKc, tmVc, tmKt,
+                            tmVt, aa);
+        }
+    } else if (p.splits > 1) {
+        le = launch_pdl_cluster(tree_attn_kernel, dim3(p.blocks * p.splits), dim3(kAttnThreads), kAttnSmem, st, p.splits,
+                                tmQ, tmKc, tmVc, tmKt, tmVt, aa);
+    } else {
+        le = launch_pdl(tree_attn_kernel, dim3(p.blocks), dim3(kAttnThreads), kAttnSmem, st, tmQ, tmKc, tmVc, tmKt, tmVt,
+                        aa);
+    }
     if (le != cudaSuccess) return DART_ERR_CUDA;
     if (ev && cudaEventRecord(ev[2], st) != cudaSuccess) return DART_ERR_CUDA;
     return DART_OK;

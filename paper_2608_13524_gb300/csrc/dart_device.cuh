@@ -35,6 +35,7 @@ __device__ __forceinline__ bool bounds_check(int* status, bool ok) {
 
 // A wait that has not completed after this long means a bug; give up.
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
+constexpr uint32_t kWaitPolls = 32;  // polls between two looks at the timer and the abort flag
 
 constexpr int kNPadMax = 256;       // max nodes per depth (nseq * W)
 constexpr int kTileM = 128;         // MMA M: vocabulary rows / output features per tile
@@ -134,11 +135,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 __device__ __forceinline__ bool mbar_wait_inline(uint64_t* bar, uint32_t parity, volatile int* abort,
                                                  unsigned long long limit_ns = kWaitLimitNs) {
     if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer_ns();
-    for (;;) {
+    unsigned long long t0 = 0;
+    for (uint32_t n = 1;; n++) {
         if (mbar_try_wait(bar, parity)) return true;
-        if (*abort) return false;
-        if (globaltimer_ns() - t0 > limit_ns) return false;
+        if (n % kWaitPolls == 0) {  // (reading the timer delays the polls)
+            if (*abort) return false;
+            const unsigned long long t = globaltimer_ns();
+            if (t0 == 0) t0 = t;
+            if (t - t0 > limit_ns) return false;
+        }
     }
 }
 __device__ __noinline__ static bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort,

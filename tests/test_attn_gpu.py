@@ -226,3 +226,22 @@ def test_tolerance_detects_a_planted_mask_error(dart, monkeypatch):
     monkeypatch.setattr(ta, "root_path", with_sibling)
     bad = oracle_attention(cfg, x)
     assert np.abs(got - bad).max() > 10 * ATOL
+
+
+# two query tiles per CTA (more query tiles than SMs): an odd number of tiles, rows past the last
+# node, tiles of different key ranges, one head per kv head and sixteen, no context, a last wave of
+# single tiles (C = 300: 168 pairs) and none
+PAIRS = [A("pair-odd", 4, 150, 70, L=8, W=24, seed=101), A("pair-fill", 5, 192, 130, L=8, W=40, seed=102, fill=0.55),
+         A("pair-g1", 3, 300, 0, L=6, W=64, seed=103, Hq=24, Hkv=24),
+         A("pair-g16", 8, 129, 257, L=16, W=9, seed=104, Hq=32, Hkv=2),
+         A("pair-waves", 7, 192, 300, L=8, W=30, seed=105)]
+
+
+@pytest.mark.parametrize("cfg", PAIRS, ids=lambda c: c.name)
+def test_attention_query_tile_pairs(dart, cfg):
+    x = make_attn_inputs(cfg)
+    got, _ = gpu_attention(dart, cfg, x)
+    g = np.random.Generator(np.random.PCG64(cfg.seed))
+    rows = [(s, int(i)) for s in range(cfg.nseq)
+            for i in {0, int(x["n_nodes"][s]) - 1, *g.integers(0, int(x["n_nodes"][s]), 12)}]
+    compare(cfg, x, got, oracle_attention(cfg, x, rows=rows), rows=rows)
