@@ -67,6 +67,14 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The two halves of a cluster barrier that orders no memory: after the second
+// every CTA of the cluster has started, so its shared memory may be accessed.
+__device__ __forceinline__ void cluster_started_arrive() {
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_started_wait() {
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
 __device__ __forceinline__ float ld_cluster_f32(uint32_t local, uint32_t rank) {
     uint32_t remote;
     float v;
@@ -131,14 +139,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 // Waits for the phase with the given parity.  Gives up (returns false) when
 // *abort becomes nonzero or after limit_ns (kWaitLimitNs unless a test asks
-// for a shorter limit).
+// for a shorter limit).  kPolls = 1 looks at the timer after every poll: the
+// fused fp32 round, where all warps of a block poll one barrier together and
+// are better kept apart.
+template <uint32_t kPolls = kWaitPolls>
 __device__ __forceinline__ bool mbar_wait_inline(uint64_t* bar, uint32_t parity, volatile int* abort,
                                                  unsigned long long limit_ns = kWaitLimitNs) {
     if (mbar_try_wait(bar, parity)) return true;
     unsigned long long t0 = 0;
     for (uint32_t n = 1;; n++) {
         if (mbar_try_wait(bar, parity)) return true;
-        if (n % kWaitPolls == 0) {  // (reading the timer delays the polls)
+        if (n % kPolls == 0) {  // (reading the timer delays the polls)
             if (*abort) return false;
             const unsigned long long t = globaltimer_ns();
             if (t0 == 0) t0 = t;

@@ -844,7 +844,7 @@ __global__ void __launch_bounds__(kRoundThreads, 1) round_cluster_f32_kernel(con
             const int g = (dep - 1) * nch + ch;
             const int st = g & 1;
             const int rows = min(CR, R - ch * CR);
-            if (!mbar_wait_inline(&sbar[st], static_cast<uint32_t>(g >> 1) & 1u, abort)) {
+            if (!mbar_wait_inline<1>(&sbar[st], static_cast<uint32_t>(g >> 1) & 1u, abort)) {
                 if (lane == 0) {
                     *abort = 1;
                     atomicOr(a.status, kDevTimeout);
@@ -1005,7 +1005,7 @@ __global__ void __launch_bounds__(kRoundThreads, 1) round_cluster_f32_kernel(con
                         : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         if (a.wres && !wready) {
-            if (!mbar_wait_inline(&sbar[2], 0u, abort) && lane == 0) {
+            if (!mbar_wait_inline<1>(&sbar[2], 0u, abort) && lane == 0) {
                 *abort = 1;
                 atomicOr(a.status, kDevTimeout);
             }
@@ -1117,8 +1117,8 @@ __global__ void __launch_bounds__(kRoundThreads, 1) round_cluster_f32_kernel(con
         // a wait gave up: the copies this block issued and did not consume
         // finish before it exits (their waits bounded again)
         int zero = 0;
-        for (int g = consumed; g < issued; g++) (void)mbar_wait_inline(&sbar[g & 1], static_cast<uint32_t>(g >> 1) & 1u, &zero);
-        if (a.wres && a.L > 1) (void)mbar_wait_inline(&sbar[2], 0u, &zero);
+        for (int g = consumed; g < issued; g++) (void)mbar_wait_inline<1>(&sbar[g & 1], static_cast<uint32_t>(g >> 1) & 1u, &zero);
+        if (a.wres && a.L > 1) (void)mbar_wait_inline<1>(&sbar[2], 0u, &zero);
     }
     cluster_sync_all();  // no block leaves while a peer may still read its shared memory
 }

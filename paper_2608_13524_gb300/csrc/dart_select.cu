@@ -114,6 +114,7 @@ __device__ __forceinline__ void append_reaching(const uint64_t* keys, int n, uin
 template <int kPer>
 __global__ void __launch_bounds__(kMergeThreads) merge_select_kernel(const SelectArgs a, int cs, int npb) {
     pdl_trigger();
+    cluster_started_arrive();
     constexpr int kNodes = kMergeThreads / kPer, kWarps = kPer / 32;
     extern __shared__ __align__(16) uint64_t survs[];  // [nh][kRankMax] keys that reach the threshold
     __shared__ __align__(16) uint64_t heads2[kNodes][kPer];  // list heads, or per-warp group maxima [kWarps][32]
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_select_kernel(const Selec
     const float2 none = make_float2(-INFINITY, 0.0f);
     const bool wide = (a.klist & 3) == 0 && (reinterpret_cast<uintptr_t>(a.part_key) & 31u) == 0;
     pdl_wait();
+    cluster_started_wait();  // block 0 runs before candidates are sent to it
     const int prev_count = a.dep == 1 ? 1 : __ldcg(a.tree_count + s * a.L + a.dep - 2);
     const uint32_t fk0 = smem_u32(fkey), ft0 = smem_u32(ftok);
 #pragma unroll 1

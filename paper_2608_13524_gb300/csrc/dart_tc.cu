@@ -215,7 +215,7 @@ __device__ __forceinline__ void mma_issuer(const Work& w, uint8_t* ring, int sta
     }
 }
 
-// ---- the same roles for a CTA pair (lmhead_pair_kernel, gemm_pair_kernel)
+// ---- the same roles for a CTA pair (lmhead_tc_kernel with kPair)
 //
 // Each CTA loads its own A tile (128 rows) and one half of the group's B
 // rows: the leader the hi rows, its peer the lo rows.  A stage is full when
