@@ -980,6 +980,8 @@ int enqueue_depth(dart_handle* h, const dart_config& c, const std::vector<DepthP
             ba.dlog_row_off = la.dlog_row_off;
             ba.ybuf = h->bound_y;
             ba.status = h->status;
+            ba.num_sms = h->num_sms;
+            ba.smem_sm = h->smem_optin;
             const int pb = prof_begin(h, kBound, st);
             e = launch_seed_score(ba, c.nseq, st);
             prof_end(h, pb, st);

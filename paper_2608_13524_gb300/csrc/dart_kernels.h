@@ -160,6 +160,7 @@ struct BoundArgs {
     long long dlog_seq_stride, dlog_row_off;
     float* ybuf;                // [nseq * P][R]
     int* status;
+    int num_sms, smem_sm;       // SMs, shared memory of one
 };
 cudaError_t launch_seed_score(const BoundArgs& a, int nseq, cudaStream_t st);
 size_t seed_score_smem(int d);
