@@ -109,12 +109,14 @@ __device__ __forceinline__ void for_row(const float* x, int V, F&& f) {
 // [V j / S, V (j + 1) / S) of the row; keys key(x, v) order by (value desc,
 // token asc).  Every block finds the exact top min(K, slice) keys of its
 // slice; the global top K is among them.  Pass 1: every thread finds the
-// largest key of its share of the slice.  Bound T: in every warp the m-th largest of these maxima
+// largest value of its share of the slice and makes a key of it.  Bound T: in every warp the m-th largest of these maxima
 // (m = ceil(K/32), warp bitonic sort), minimised over the warps -- at least
 // 32*m >= K threads hold a key >= T, so the K-th largest key is >= T, and
 // only a small multiple of K keys reach it.  Pass 2 gathers the keys >= T
 // (the slice is now in L2) and the top K of them are ranked in shared
-// memory.  If more than kCollCap keys reach T (pathological rows, e.g. many
+// memory.  Both passes compare floats (with one block per row the instructions
+// per element bound them: 128 rows of 151936, K = 64, on GB300: 40.9 µs with a
+// key made and compared for every element, 34.1 now).  If more than kCollCap keys reach T (pathological rows, e.g. many
 // equal values), an exact radix select over the slice decides instead: 12
 // bits per pass from the top, the keys above the threshold digit taken, and
 // once the threshold digit holds at most kCollCap keys they are gathered for
@@ -146,12 +148,16 @@ __global__ void __launch_bounds__(kTopkThreads)
     const float* x = dlog + static_cast<size_t>(row) * V + v0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) cnt[0] = cnt[1] = 0;
-    // pass 1: this thread's largest key
-    uint64_t mx = 0ull;
+    // pass 1: the key of this thread's largest value (any of its keys would do for the bound)
+    float best = 0.0f;
+    int at = -1;
     for_row(x, Vs, [&](float xv, int v) {
-        const uint64_t k = make_key(xv, static_cast<uint32_t>(v0 + v));
-        mx = k > mx ? k : mx;
+        if (at < 0 || xv > best) {
+            best = xv;
+            at = v;
+        }
     });
+    const uint64_t mx = at < 0 ? 0ull : make_key(best, static_cast<uint32_t>(v0 + at));
     {
         const int m = (Kl + 31) / 32;
         uint64_t hv = mx;
@@ -172,7 +178,9 @@ __global__ void __launch_bounds__(kTopkThreads)
     uint64_t T = wmin[0];
     for (int w = 1; w < kTopkThreads / 32; w++) T = wmin[w] < T ? wmin[w] : T;
     // pass 2: gather every key >= T
+    const float tv = key_val(T);
     for_row(x, Vs, [&](float xv, int v) {
+        if (xv < tv) return;  // (a NaN on either side is left to the keys)
         const uint64_t k = make_key(xv, static_cast<uint32_t>(v0 + v));
         if (k >= T) {
             const int pos = atomicAdd(&cnt[1], 1);
