@@ -83,6 +83,11 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t local, uint32_t rank) {
     return v;
 }
 
+__device__ __forceinline__ void st_cluster_s32(uint32_t local, uint32_t rank, int v) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
+}
 __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t local, uint32_t rank) {
     uint32_t remote;
     float4 v;
@@ -135,6 +140,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "=r"(ok)
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
+    return ok != 0;
+}
+// The same without the wait that try_wait may make.
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok)
+                 : "r"(smem_u32(bar)), "r"(parity)
+                 : "memory");
     return ok != 0;
 }
 // Waits for the phase with the given parity.  Gives up (returns false) when

@@ -53,11 +53,6 @@ __device__ __forceinline__ void st_cluster_u64(uint32_t local, uint32_t rank, ui
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(remote), "l"(v) : "memory");
 }
-__device__ __forceinline__ void st_cluster_s32(uint32_t local, uint32_t rank, int v) {
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
-    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
-}
 
 // More than kRankMax keys reach the threshold (many equal scores): the kk
 // largest of the n keys by radix select, into surv (unsorted).

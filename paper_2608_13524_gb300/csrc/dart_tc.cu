@@ -221,6 +221,12 @@ __device__ __forceinline__ void mma_issuer(const Work& w, uint8_t* ring, int sta
 // rows: the leader the hi rows, its peer the lo rows.  A stage is full when
 // all four copies have completed on the leader's barrier; it is empty when
 // the leader's commit has arrived in both CTAs.
+//
+// A commit arrives in the peer's shared memory some time after the MMAs it
+// tracks, and no barrier of threads orders that.  So every arrival is waited
+// for where it lands, before the CTA leaves: the last ones of `empty` by the
+// CTA's producer, that of an accumulator its epilogue does not read by the
+// epilogue's first thread.
 
 template <int NG>
 struct PairLayout {
@@ -273,18 +279,20 @@ __device__ __forceinline__ void producer_pair(const CUtensorMap* tmA, const CUte
             phase ^= 1u;
         }
     }
-    if (!ok) {
-        // copies still in flight must land before the pair leaves: the
-        // leader's barriers track both CTAs'; the peer, which cannot wait on
-        // them, stays a millisecond, far longer than a copy takes
-        if (rank == 0) {
-            const uint32_t first = fills > static_cast<uint32_t>(stages) ? fills - stages : 0;
-            for (uint32_t f = first; f < fills; f++) drain_wait(&full[f % stages], (f / stages) & 1u);
-        } else {
-            const unsigned long long t0 = globaltimer_ns();
-            while (globaltimer_ns() - t0 < 1000000ull) {
-            }
+    // the fills that no later fill waited for
+    const uint32_t first = fills > static_cast<uint32_t>(stages) ? fills - stages : 0;
+#pragma unroll 1
+    for (uint32_t f = first; f < fills && ok; f++) {
+        if (!mbar_wait(&empty[f % stages], (f / stages) & 1u, abort)) {
+            record_timeout(status, abort);
+            ok = false;
         }
+    }
+    // copies still in flight must land before the pair leaves: the leader's
+    // barriers track both CTAs' (the peer, which cannot wait on them, stays
+    // with it: teardown)
+    if (!ok && rank == 0) {
+        for (uint32_t f = first; f < fills; f++) drain_wait(&full[f % stages], (f / stages) & 1u);
     }
 }
 
@@ -337,7 +345,7 @@ __device__ __forceinline__ void mma_issuer_pair(const Work& w, uint8_t* ring, in
 struct Smem {
     uint8_t* ring;
     uint64_t *full, *empty, *tfull, *tempty, *tdown;
-    int* misc;  // [0] tmem base, [1] abort flag, [2] epilogue flag
+    int* misc;  // [0] tmem base, [1] abort flag, [2] epilogue flag, [3] pairs: the other CTA's abort flag
     uint8_t* tail;
 };
 
@@ -372,6 +380,7 @@ __device__ __forceinline__ uint32_t setup(const Smem& s, int stages, int ncols, 
         mbar_init(s.tdown, 1);
         s.misc[1] = 0;
         s.misc[2] = 0;
+        s.misc[3] = 0;
         fence_mbar_init();
     }
     if (warp == 1) {
@@ -390,14 +399,47 @@ __device__ __forceinline__ uint32_t setup(const Smem& s, int stages, int ncols, 
     return static_cast<uint32_t>(s.misc[0]);
 }
 
+// Debug builds: every phase of this CTA's `empty` and `tfull` barriers that
+// the pair's commits end has ended when its threads are done (unless a wait
+// gave up).
+__device__ __forceinline__ void check_pair_quiet(const Smem& s, const Work& w, int stages, int nacc, int* status) {
+#ifdef DART_DEBUG
+    __syncthreads();
+    if (threadIdx.x != 0 || s.misc[1] != 0) return;
+    const int fills = w.ntiles * (w.kb1 - w.kb0);
+    bool quiet = true;
+    for (int f = max(fills - stages, 0); f < fills; f++)
+        quiet = mbar_test_wait(&s.empty[f % stages], static_cast<uint32_t>(f / stages) & 1u) && quiet;
+    for (int i = max(w.ntiles - nacc, 0); i < w.ntiles; i++)
+        quiet = mbar_test_wait(&s.tfull[i % nacc], static_cast<uint32_t>(i / nacc) & 1u) && quiet;
+    bounds_check(status, quiet);
+#endif
+}
+
 template <bool kPair = false>
-__device__ __forceinline__ void teardown(uint32_t tmem_base, int ncols) {
+__device__ __forceinline__ void teardown(uint32_t tmem_base, int ncols, int* misc = nullptr) {
     tc_fence_before();
     __syncthreads();
-    if constexpr (kPair) cluster_sync_all();  // neither CTA leaves while the other may still signal it
+    if constexpr (kPair) {
+        // neither CTA leaves while the other's threads may still signal it,
+        // and neither frees the TMEM that its MMAs write
+        if (threadIdx.x == 0) st_cluster_s32(smem_u32(&misc[3]), cluster_ctarank() ^ 1u, misc[1]);
+        cluster_sync_all();
+    }
     if ((threadIdx.x >> 5) == 1) {
         __syncwarp();
         tc_fence_after();
+        if constexpr (kPair) {
+            // A wait gave up in one of the two: copies and arrivals that were
+            // not waited for land within a millisecond (the leader has issued
+            // its last commit and seen it complete before the barrier).
+            if (misc[1] != 0 || misc[3] != 0) {
+                const unsigned long long t0 = globaltimer_ns();
+                while (globaltimer_ns() - t0 < 1000000ull) {
+                }
+            }
+            __syncwarp();
+        }
         if constexpr (kPair) tmem_dealloc_pair(tmem_base, ncols);
         else tmem_dealloc(tmem_base, ncols);
     }
@@ -636,8 +678,15 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
 #pragma unroll
         for (int ci = 0; ci < kChunks; ci++) epi_stash(e, NG, quarter, lane, ((wi >> 2) + 4 * ci) * 16, ssum[ci]);
         epi_finalize(e, NG, a.k, etid, kEpi, g * NG, a.N, vr, a.nV, a.part_ms, a.part_key);
+        if constexpr (kPair) {
+            // the accumulator of the longer range's last tile is not read here, but its commit arrives here too
+            if (etid == 0 && own < w.ntiles && s.misc[2] != 0 &&
+                !mbar_wait(&s.tfull[own % kNacc], (own / kNacc) & 1, abort))
+                record_timeout(a.status, abort);
+        }
     }
-    teardown<kPair>(tmem_base, lm_tmem_cols<NG>());
+    if constexpr (kPair) check_pair_quiet(s, w, stages, kNacc, a.status);
+    teardown<kPair>(tmem_base, lm_tmem_cols<NG>(), s.misc);
 }
 
 // --------------------------------------------------------------- GEMM kernel
