@@ -61,6 +61,11 @@ typedef struct {
  * invalid configuration. */
 size_t dart_tree_attention_workspace(const dart_attn_config *cfg);
 
+/* Test hook (host only): query tiles per CTA, 1 or 2, that
+ * dart_tree_attention takes for `cfg` on a device of num_sms SMs; the output
+ * is the same.  0 on an invalid configuration. */
+int dart_tree_attention_tiles(const dart_attn_config *cfg, int num_sms);
+
 /* One tree-attention layer (see above).  Layouts, all row-major bf16 unless
  * stated, innermost dimension last:
  *   q       [nseq][B][Hq][dh]    queries of the tree rows, not rotated

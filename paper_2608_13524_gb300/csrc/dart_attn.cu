@@ -22,8 +22,8 @@
 //                      that merge their partial (max, sum, O) over
 //                      distributed shared memory, in rank order;
 //   tree_attn2_kernel  the same for two query tiles per CTA, when there are
-//                      more query tiles than SMs (and tree_attn_kernel for
-//                      what its last wave would leave);
+//                      more query tiles than SMs and pairs_pay says so (and
+//                      tree_attn_kernel for what its last wave would leave);
 // and dart_ancestor_mask's own kernel, one block per sequence.
 // tree_attn_kernel, 320 threads: warp 0 TMA producer (K ring 3 stages, V ring
 // 3 stages), warp 1 TMEM allocator + single-thread MMA issuer, warps 2-9 two
@@ -1257,6 +1257,8 @@ int pick_splits(int blocks, int max_tiles, int nsm) {
     return sp;
 }
 
+int key_tiles(const dart_attn_config& c) { return (c.C + kKeys - 1) / kKeys + (c.B + kKeys - 1) / kKeys; }
+
 Plan make_plan(const dart_attn_config* c, int nsm) {
     Plan p;
     p.G = c->Hq / c->Hkv;
@@ -1265,8 +1267,49 @@ Plan make_plan(const dart_attn_config* c, int nsm) {
     p.blocks = c->nseq * c->Hkv * p.nqt;
     p.mw = (c->B + 63) / 64;
     p.nct = (c->C + kKeys - 1) / kKeys;
-    p.splits = pick_splits(p.blocks, p.nct + (c->B + kKeys - 1) / kKeys, nsm);
+    p.splits = pick_splits(p.blocks, key_tiles(*c), nsm);
     return p;
+}
+
+// Units of the pair route that go to tree_attn_kernel, one query tile per CTA:
+// a last wave that would leave half of the SMs idle.  Measured on GB300, 512
+// pairs on 152 SMs (8 x 512 rows, 2048 context keys): four waves of pairs
+// 175 µs, three and 112 single tiles 163.
+int pair_tail(int nunits, int nsm) {
+    const int rem = nunits % nsm;
+    return nunits > nsm && 2 * rem <= nsm ? rem : 0;
+}
+
+// Whether two query tiles per CTA (tree_attn2_kernel) take less time than one:
+// with more tiles than SMs both run in waves, and a kv head with an odd number
+// of tiles leaves a pair with one (all such units come first).  In units of one
+// key tile a CTA with one query tile takes 4 + n for n key tiles, one with two
+// 3 + 1.85 n, one with two of which one is empty 5 + 1.7 n (while those run,
+// every SM streams another head's keys and values); the list schedule of the
+// pairs against the waves of the single tiles.  The five constants are fitted
+// to 530 calls timed both ways on GB300 (40 to 360 kv heads, 2 to 11 tiles
+// each, 0 to 8192 context keys): the choice costs at most 3.4 % against the
+// better side, 0.05 % on average, where pairs for all of them cost up to 37 %
+// (µs, pairs and single tiles: 40 heads of 7 tiles, 2048 keys 74.4, 57.9; 88
+// of 3 72.3, 57.3; 360 of 1 109, 99; 56 of 3 47, 54; 64 of 16 163, 190).
+bool pairs_pay(const Plan& p, int nheads, int nkt, int nsm) {
+    if (p.splits != 1 || p.blocks <= nsm || p.nqt < 2) return false;
+    const double one = 4.0 + nkt, full = (3.0 + 1.85 * nkt) / one, half = (5.0 + 1.7 * nkt) / one;
+    const int nunits = nheads * ((p.nqt + 1) / 2), tail = pair_tail(nunits, nsm);
+    const int nhalf = p.nqt % 2 ? std::min(nheads, nunits - tail) : 0, nfull = nunits - tail - nhalf;
+    // the half-empty units: nb SMs are done with them at t1, the others at t0
+    const int nb = nhalf % nsm;
+    const double t0 = nhalf / nsm * half, t1 = t0 + half;
+    double end = 1e30;
+    for (int i = std::max(0, nfull / nsm - 2); i <= nfull / nsm + 3; i++) {
+        for (const double t : {t0 + i * full, t1 + i * full}) {
+            if (t < (nb > 0 ? t1 : t0) - 1e-9) continue;
+            const double done = (nsm - nb) * std::floor((t - t0) / full + 1e-9) +
+                                nb * std::max(0.0, std::floor((t - t1) / full + 1e-9));
+            if (done >= nfull) end = std::min(end, t);
+        }
+    }
+    return end + (tail > 0 ? 1.0 : 0.0) < static_cast<double>((p.blocks + nsm - 1) / nsm);
 }
 
 WsLayout ws_layout(const dart_attn_config* c) {
@@ -1395,7 +1438,7 @@ int enqueue_tree_attention(const dart_attn_config* cfg, const void* q, const voi
     __nv_bfloat16* kr = reinterpret_cast<__nv_bfloat16*>(ws + wl.off_kr);
     float2* cs = reinterpret_cast<float2*>(ws + wl.off_cs);
 
-    const bool two = p.splits == 1 && p.blocks > nsm;  // two query tiles per CTA (tree_attn2_kernel)
+    const bool two = pairs_pay(p, c.nseq * c.Hkv, key_tiles(c), nsm);  // two query tiles per CTA (tree_attn2_kernel)
     CUtensorMap tmQ, tmKc, tmVc, tmKt, tmVt, tmO;
     if (two && !encode_out(&tmO, out, c.nseq, c.B, c.Hq, p.G, p.qpt)) return DART_ERR_CUDA;
     if (!encode_q(&tmQ, q, c.nseq, c.B, c.Hq, p.G, p.qpt)) return DART_ERR_CUDA;
@@ -1450,12 +1493,7 @@ int enqueue_tree_attention(const dart_attn_config* cfg, const void* q, const voi
     if (ev && cudaEventRecord(ev[1], st) != cudaSuccess) return DART_ERR_CUDA;
     cudaError_t le;
     if (two) {
-        // Whole waves of pairs; a last wave that would leave half of the SMs
-        // idle goes to tree_attn_kernel, one query tile per CTA.  Measured on
-        // GB300, 512 pairs on 152 SMs (8 x 512 rows, 2048 context keys): four
-        // waves of pairs 175 µs, three and 112 single tiles 163.
-        const int rem = aa.nunits % nsm;
-        const int single = aa.nunits > nsm && 2 * rem <= nsm ? rem : 0;
+        const int single = pair_tail(aa.nunits, nsm);
         le = launch_pdl(tree_attn2_kernel, dim3(aa.nunits - single), dim3(kAttn2Threads), kAttn2Smem, st, tmQ, tmKc, tmVc,
                         tmKt, tmVt, tmO, aa);
         if (le == cudaSuccess && single > 0) {
@@ -1487,6 +1525,11 @@ size_t dart_tree_attention_workspace(const dart_attn_config* cfg) {
     return ws_layout(cfg).total;
 }
 
+
+int dart_tree_attention_tiles(const dart_attn_config* cfg, int num_sms) {
+    if (!valid_cfg(cfg) || num_sms < 1) return 0;
+    return pairs_pay(make_plan(cfg, num_sms), cfg->nseq * cfg->Hkv, key_tiles(*cfg), num_sms) ? 2 : 1;
+}
 
 int dart_tree_attention(const dart_attn_config* cfg, const void* q, const void* k_tree, const void* v_tree,
                         const void* k_ctx, const void* v_ctx, const int32_t* pos_ids, const uint64_t* mask,

@@ -105,6 +105,7 @@ def lib():
                                         C.c_size_t, vp, vp]),
             "dart_tree_attention_timed": (i, [C.POINTER(DartAttnConfig), vp, vp, vp, vp, vp, vp, vp, vp, vp, vp,
                                               C.c_size_t, vp, C.POINTER(f), C.POINTER(f), vp]),
+            "dart_tree_attention_tiles": (i, [C.POINTER(DartAttnConfig), i]),
             "dart_ancestor_mask": (i, [vp, vp, i, i, vp, vp]),
             "dart_destroy": (None, [vp]),
             "dart_status_string": (C.c_char_p, [i]),
@@ -388,6 +389,11 @@ def make_attn_config(nseq, B, C_ctx, Hq, Hkv, dh, rope_theta, scale) -> DartAttn
 
 def dart_tree_attention_workspace(acfg: DartAttnConfig) -> int:
     return int(lib().dart_tree_attention_workspace(C.byref(acfg)))
+
+
+def dart_tree_attention_tiles(acfg: DartAttnConfig, num_sms: int) -> int:
+    """Query tiles per CTA that the layer takes on a device of num_sms SMs."""
+    return int(lib().dart_tree_attention_tiles(C.byref(acfg), int(num_sms)))
 
 
 def dart_tree_attention(acfg: DartAttnConfig, q, k_tree, v_tree, k_ctx, v_ctx, pos_ids, mask, n_nodes, out,

@@ -245,3 +245,19 @@ def test_attention_query_tile_pairs(dart, cfg):
     rows = [(s, int(i)) for s in range(cfg.nseq)
             for i in {0, int(x["n_nodes"][s]) - 1, *g.integers(0, int(x["n_nodes"][s]), 12)}]
     compare(cfg, x, got, oracle_attention(cfg, x, rows=rows), rows=rows)
+
+
+# more query tiles than SMs, one or three tiles per kv head: single tiles (ONE), and pairs whose
+# second tile is empty for every head (TWO)
+ONE_OR_THREE = [A("one-tile", 20, 32, 70, L=4, W=12, seed=111), A("three-tiles", 11, 96, 40, L=8, W=16, seed=112),
+                A("three-tiles-pairs", 7, 70, 200, L=8, W=16, seed=113, fill=0.9)]
+
+
+@pytest.mark.parametrize("cfg", ONE_OR_THREE, ids=lambda c: c.name)
+def test_attention_odd_tiles_per_head(dart, cfg):
+    x = make_attn_inputs(cfg)
+    got, _ = gpu_attention(dart, cfg, x)
+    g = np.random.Generator(np.random.PCG64(cfg.seed))
+    rows = [(s, int(i)) for s in range(cfg.nseq)
+            for i in {0, int(x["n_nodes"][s]) - 1, *g.integers(0, int(x["n_nodes"][s]), 6)}]
+    compare(cfg, x, got, oracle_attention(cfg, x, rows=rows), rows=rows)
