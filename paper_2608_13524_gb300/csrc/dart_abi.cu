@@ -1325,8 +1325,10 @@ SeqHeapArgs seq_heap_args(const dart_handle* h, const float* anchor, const dart_
     return a;
 }
 
-// Scoring of the pass's targets, the best Bp children of each into its entry.
-int enqueue_seq_score(dart_handle* h, const float* dlog, const float* h32, cudaStream_t st) {
+// Scoring of the pass's targets, the best Bp children of each into its entry
+// (may_idle: the pass may have none; with one target a pass few have none, and
+// the look at them would cost each 1 %).
+int enqueue_seq_score(dart_handle* h, const float* dlog, const float* h32, bool may_idle, cudaStream_t st) {
     const dart_config& cc = h->ccfg;
     const DepthPlan& p = h->splans[2];
     LmheadArgs la = lmhead_args(h, cc, p, dlog, h32);
@@ -1336,6 +1338,7 @@ int enqueue_seq_score(dart_handle* h, const float* dlog, const float* h32, cudaS
     la.dlog_row = h->sh_dlog_row;
     la.zout = h->sh_zrow;
     la.zout_stride = cc.V;
+    la.row_ent = may_idle && h->sh_M > 1 ? h->sh_row_ent : nullptr;
     int pi = prof_begin(h, kLmhead, st);
     cudaError_t e = h->wdtype == DART_BF16 ? launch_lmhead_tc(&h->tmE, &h->tmH[ng_index(p.NG)], la, p.smem, st)
                                            : launch_lmhead_f32(la, st);
@@ -1367,7 +1370,7 @@ int enqueue_seq_begin(dart_handle* h, const float* dlog, const SeqHeapArgs& a, c
     const cudaError_t e = launch_seqheap_init(a, st);
     prof_end(h, pi, st);
     if (e != cudaSuccess) return DART_ERR_CUDA;
-    int rc = enqueue_seq_score(h, dlog, h->hbuf[0], st);
+    int rc = enqueue_seq_score(h, dlog, h->hbuf[0], false, st);
     if (rc == DART_OK) rc = enqueue_seq_step(h, a, cond, has_cond, st);
     return rc;
 }
@@ -1376,7 +1379,7 @@ int enqueue_seq_begin(dart_handle* h, const float* dlog, const SeqHeapArgs& a, c
 int enqueue_seq_pass(dart_handle* h, const float* dlog, const SeqHeapArgs& a, cudaGraphConditionalHandle cond,
                      bool has_cond, cudaStream_t st) {
     int rc = enqueue_head_update(h, h->ccfg, h->splans[2], h->hbuf[0], h->hbuf[1], false, st);
-    if (rc == DART_OK) rc = enqueue_seq_score(h, dlog, h->hbuf[1], st);
+    if (rc == DART_OK) rc = enqueue_seq_score(h, dlog, h->hbuf[1], !has_cond, st);
     if (rc == DART_OK) rc = enqueue_seq_step(h, a, cond, has_cond, st);
     return rc;
 }

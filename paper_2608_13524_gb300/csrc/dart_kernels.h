@@ -101,6 +101,7 @@ struct LmheadArgs {
     const int* dlog_row;  // [N / P] drafter row of each sequence's nodes (replaces dlog_row_off / V)
     float* zout;          // z[n][v] written to zout[n * zout_stride + v] (node groups <= 64)
     long long zout_stride;
+    const int* row_ent;   // [N] fp32 kernel: nothing is done when no row has a value >= 0
     const float* seed_y;  // [N][seed_R] seed scores (launch_seed_score): the filter starts from each
     int seed_R;           // node's k-th largest, which is also published into gthr (null: no seed pass)
 };

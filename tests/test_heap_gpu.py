@@ -215,3 +215,31 @@ def test_seq_heap_passes(dart, nseq, V, L, B, wdtype):
         assert dart.dart_status_sync(eng.h) == 0
     finally:
         eng.close()
+
+
+def test_idle_passes_do_not_score(dart):
+    """As a fixed launch sequence the fp32 search launches B - 1 passes, of
+    which few have a prefix to correct: the others' LM-head streams no E.
+    (Bound: with B = 2 both passes score; of the forty of B = 40 a search of
+    depth 4 that corrects four prefixes a pass needs well under half.)"""
+    per_launch = {}
+    for B in (2, 40):
+        cfg = Config("heap-idle", 1, 60000, 512, 4, 2, 2, B, "f32", 0.0, 76, variants=2)
+        x = make_inputs(cfg)
+        dx = to_device(cfg, x)
+        eng = dart.Dart(cfg, dx["Wi"], dx["Wo"], dx["E"])
+        try:
+            g = tree_to_numpy(eng.build_seq_heap(dx["Dlog"], dx["h0"]))
+            dart.dart_set_profiling(eng.h, True)
+            eng.build_seq_heap(dx["Dlog"], dx["h0"])
+            dart.dart_profile_read_kinds(eng.h)
+            p = tree_to_numpy(eng.build_seq_heap(dx["Dlog"], dx["h0"]))
+            ms, launches = dart.dart_profile_read_kinds(eng.h)["lmhead"]
+            for k in g:
+                np.testing.assert_array_equal(p[k], g[k], err_msg=k)
+            assert dart.dart_status_sync(eng.h) == 0
+        finally:
+            eng.close()
+        assert launches == B
+        per_launch[B] = ms / launches
+    assert per_launch[40] < 0.625 * per_launch[2], per_launch
