@@ -522,17 +522,24 @@ int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, st
                         g->S = std::max(1, std::min(g->KB, cap / tiles_mg));
                     }
                 }
-                // A grid of at most one CTA per SM: all of an SM's shared
-                // memory for its pipeline (the loads in flight, not the
-                // tensor cores, bound a CTA that walks a long k range).
-                // Measured on GB300, 256 nodes, d = 4096 (128 CTAs of 64
-                // k-blocks): 3 stages 34.1 us per GEMM and 1289 us per
-                // round of 8 x 32 nodes with K = 64, 7 stages 30.0 and 1179.
+                // A grid of at most one CTA per SM takes all of an SM's shared
+                // memory for its stages, if its clusters still all fit.  (On
+                // GB300 they do: cudaOccupancyMaxActiveClusters counts one
+                // CTA per SM at either size, 15 clusters of 8 and 23 of 6, so
+                // 17 to 19 row tiles split k by 6.)  This acts on groups of at
+                // most 32 nodes (64: already one CTA per SM, seven stages) and
+                // matters little: measured on GB300, us per round with and
+                // without, 32 children, d = 2304 473.4 and 477.0, d = 1024 with
+                // K = 64 176.4 and 177.8, d = 2112 to 2432 with K = 64 206.3 and
+                // 203.5, 8 x 32 nodes with K = 64 1146 and 1147.
                 for (GemmArgs* g : {&p.g1, &p.g2}) {
                     int& sm = g == &p.g1 ? p.g1_smem : p.g2_smem;
                     const int sbg = tc_stage_bytes(g->NG);
-                    if (g->MT * g->G * g->S <= h->num_sms)
-                        g->stages = std::min(tc_stages(h->smem_optin, sbg, gemm_tc_fixed_smem(16)), 8);
+                    const int st1 = std::min(tc_stages(h->smem_optin, sbg, gemm_tc_fixed_smem(16)), 8);
+                    const bool cl = g == &p.g1 ? cluster1 : cluster;
+                    if (g->MT * g->G * g->S <= h->num_sms &&
+                        (!cl || gemm_tc_max_clusters(g->NG, gemm_tc_fixed_smem(st1) + st1 * sbg, g->S) >= g->MT * g->G))
+                        g->stages = st1;
                     sm = gemm_tc_fixed_smem(g->stages) + g->stages * sbg;
                 }
                 p.g1.mode = cluster1 ? (p.split ? kGemmSum : kGemmSiluSplit) : kGemmPartials;
