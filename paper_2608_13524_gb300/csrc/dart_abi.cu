@@ -459,7 +459,7 @@ int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, st
         p.klist = c.cand_k > 0 ? 1 : c.k;
         p.cand_ds = 0;
         if (c.cand_k > 0) {
-            p.cand_ds = cand_score_slices(p.P, c.d, c.nseq, c.cand_k, h->smem_optin);
+            p.cand_ds = cand_score_slices(p.P, c.d, c.nseq, c.cand_k, h->smem_optin - 1024);
             if (p.cand_ds == 0) return DART_ERR_UNSUPPORTED;
         }
         p.Pn = caps[dep];
@@ -720,7 +720,7 @@ int alloc_workspace(dart_handle* h) {
     if (select_set_smem_limits() != cudaSuccess) return DART_ERR_CUDA;
     if (c.cand_k > 0) {
         for (int dep = 1; dep <= c.L; dep++)
-            if (h->plans[dep].P * (c.d / h->plans[dep].cand_ds) * 4 > h->smem_optin - 1024)
+            if (cand_score_smem(c.nseq, h->plans[dep].P, c.d, h->plans[dep].cand_ds) > h->smem_optin - 1024)
                 return DART_ERR_UNSUPPORTED;
         if (cudaMemset(h->cand_rticket, 0, static_cast<size_t>(c.nseq) * c.L * sizeof(int)) != cudaSuccess)
             return DART_ERR_CUDA;

@@ -469,8 +469,11 @@ int cand_topk_slices(int V, int K, int rows, int num_sms) {
 }
 
 int cand_score_slices(int P, int d, int nseq, int K, int max_smem) {
-    // slices of d per block: enough blocks to spread the loads (>= 128), the
-    // staged slice within 64 KB, and d / DS a multiple of 4 floats
+    // Slices of d: enough (slice, group of 8 candidates) units to spread the
+    // loads (>= 128; with kScoreManyNodes nodes the groups are of 16), a slice
+    // of all P states within 64 KB, and d / DS a multiple of 4 floats.  A
+    // slice of all P states above max_smem (d = 64 * an odd number, large) is
+    // not supported, although the kernel stages PC of them at a time.
     const int ngroups = (K + kScoreWarps - 1) / kScoreWarps;
     int DS = 1;
     while (d % (8 * DS) == 0 &&
@@ -514,15 +517,31 @@ cudaError_t launch_row_topk_by_value(const float* x, int rows, int V, int K, int
                       part, ticket, 1, out_stride, val, out_row);
 }
 
+// Candidates per group, blocks per cluster, node states staged at a time, and
+// the shared memory of both these and the partial sums (at most 83 KB for any
+// supported shape).
+struct ScorePlan {
+    bool many;
+    int G, cs, PC, smem;
+};
+static ScorePlan score_plan(int nseq, int P, int d, int DS) {
+    ScorePlan p;
+    p.many = nseq * P >= kScoreManyNodes;
+    p.G = p.many ? 16 : 8;
+    p.cs = std::min(DS, kScoreCluster);  // (DS is a power of two)
+    const int dchunk = d / DS;
+    p.PC = std::max(1, std::min(P, kScoreStage / (dchunk * 4)));
+    p.smem = (p.PC * dchunk + DS / p.cs * (p.G + 1) * P) * 4;
+    return p;
+}
+
+int cand_score_smem(int nseq, int P, int d, int DS) { return score_plan(nseq, P, d, DS).smem; }
+
 cudaError_t launch_cand_score(const CandArgs& a, cudaStream_t st) {
-    const bool many = a.nseq * a.P >= kScoreManyNodes;
-    const int G = many ? 16 : 8, ngroups = (a.K + G - 1) / G;
-    const int cs = std::min(a.DS, kScoreCluster);  // (DS is a power of two)
-    const int dchunk = a.d / a.DS;
-    const int PC = std::max(1, std::min(a.P, kScoreStage / (dchunk * 4)));
-    const int smem = (PC * dchunk + a.DS / cs * (G + 1) * a.P) * 4;
-    return launch_pdl_cluster(score_kernel(a.wbf16 != 0, many), dim3(a.nseq * ngroups * cs), dim3(kScoreThreads), smem,
-                              st, cs, a, cs, PC);
+    const ScorePlan p = score_plan(a.nseq, a.P, a.d, a.DS);
+    const int ngroups = (a.K + p.G - 1) / p.G;
+    return launch_pdl_cluster(score_kernel(a.wbf16 != 0, p.many), dim3(a.nseq * ngroups * p.cs), dim3(kScoreThreads),
+                              p.smem, st, p.cs, a, p.cs, p.PC);
 }
 
 }  // namespace dart

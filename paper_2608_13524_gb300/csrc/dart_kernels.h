@@ -252,7 +252,8 @@ cudaError_t launch_row_topk_by_value(const float* x, int rows, int V, int K, int
 int cand_topk_slices(int V, int K, int rows, int num_sms);
 cudaError_t launch_cand_score(const CandArgs& a, cudaStream_t st);
 int cand_topk_smem(int K);
-int cand_score_slices(int P, int d, int nseq, int K, int max_smem);  // 0: does not fit
+int cand_score_slices(int P, int d, int nseq, int K, int max_smem);  // 0: not supported
+int cand_score_smem(int nseq, int P, int d, int DS);  // dynamic shared memory of a launch
 cudaError_t cand_set_smem_limits();    // the device maximum for both kernels
 
 struct EmitArgs {
