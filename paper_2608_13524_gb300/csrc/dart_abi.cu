@@ -874,7 +874,6 @@ LmheadArgs lmhead_args(const dart_handle* h, const dart_config& c, const DepthPl
 SelectArgs select_args(const dart_handle* h, const dart_config& c, const DepthPlan& p, int dep) {
     SelectArgs sa;
     std::memset(&sa, 0, sizeof sa);
-    sa.N = p.N;
     sa.P = p.P;
     sa.k = c.k;
     sa.nV = p.nlist;

@@ -465,16 +465,13 @@ constexpr int kRankMax = 1024;  // candidate count up to which an O(n^2 / thread
 // Writes the kk largest nonzero keys, in descending order, to out[0..kk).
 // `keys` holds nlists lists of `len` keys, each sorted in descending order
 // with zeros (empty slots) last; at least kk keys are nonzero.  Only keys
-// >= a threshold T can be among the kk largest, where T is the larger of
-// `bound` (0, or a key known to have kk keys >= it, such as the largest
-// k-th key any LM-head CTA published for the node) and the kk-th largest
-// list head (some kk lists reach it; skipped when rank_heads is false); the
-// survivors are ranked by counting.
+// >= a threshold T can be among the kk largest, where T is the kk-th largest
+// list head (some kk lists reach it); the survivors are ranked by counting.
 // A block-wide radix select handles a survivor set larger than kRankMax.
 // `surv` has kRankMax slots.  Every thread of the block must call this.
 __device__ __forceinline__ void topk_of_sorted_lists(const uint64_t* keys, int nlists, int len, int kk,
-                                                     uint64_t bound, uint64_t* out, uint64_t* surv, uint64_t* thr,
-                                                     uint32_t* hist, int* scal, bool rank_heads = true) {
+                                                     uint64_t* out, uint64_t* surv, uint64_t* thr, uint32_t* hist,
+                                                     int* scal) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int n = nlists * len;
     if (tid == 0) {
@@ -482,7 +479,7 @@ __device__ __forceinline__ void topk_of_sorted_lists(const uint64_t* keys, int n
         scal[2] = 0;
     }
     __syncthreads();
-    if (rank_heads && nlists >= kk && nlists > 1) {
+    if (nlists >= kk && nlists > 1) {
         for (int r = tid; r < nlists; r += nt) {
             const uint64_t h = keys[r * len];
             if (h == 0ull) continue;
@@ -497,7 +494,7 @@ __device__ __forceinline__ void topk_of_sorted_lists(const uint64_t* keys, int n
         }
         __syncthreads();
     }
-    const uint64_t T = *thr > bound ? *thr : bound;
+    const uint64_t T = *thr;
     for (int i = tid; i < n; i += nt) {
         const uint64_t x = keys[i];
         if (x != 0ull && x >= T) {

@@ -1,5 +1,5 @@
 // Frontier selection of one depth (Algorithm 1, "retain the global top-W"),
-// shared by the selection kernels: the candidates (p, j) of sequence s are
+// for the grid form of the fused fp32 round: the candidates (p, j) of sequence s are
 // the k best children of each of its prev_count parents (node_logq /
 // node_tok, rows s*P + p, each sorted by log q~), scored by Eq. 5,
 // s = s_parent + log q~ + beta; the top W by (score desc, parent slot asc,
@@ -33,7 +33,7 @@ __device__ __forceinline__ void select_frontier(const SelectArgs& a, int s, int 
     }
     const int nvalid = block_sum_int(valid, redi);
     const int cnt = min(a.W, nvalid);
-    if (cnt > 0) topk_of_sorted_lists(keys, prev_count, a.k, cnt, 0ull, top, surv, thr, hist, scal);
+    if (cnt > 0) topk_of_sorted_lists(keys, prev_count, a.k, cnt, top, surv, thr, hist, scal);
     const size_t tb = (static_cast<size_t>(s) * a.L + a.dep - 1) * a.W;
     for (int r = tid; r < a.W; r += static_cast<int>(blockDim.x)) {
         if (r < cnt) {

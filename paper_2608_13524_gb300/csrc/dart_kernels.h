@@ -200,7 +200,7 @@ cudaError_t f32_set_smem_limits(int max_dyn);
 struct SelectArgs {
     // nV sorted key lists of klist keys per node (LM-head CTAs, or one key
     // per candidate of C_d); Pn = max |S_dep| (child slots per sequence)
-    int N, P, k, nV, klist, W, L, nseq, dep, Pn;
+    int P, k, nV, klist, W, L, nseq, dep, Pn;
     float beta;
     const float2* part_ms;
     const uint64_t* part_key;

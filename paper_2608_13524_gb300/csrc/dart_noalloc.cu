@@ -204,7 +204,6 @@ extern "C" int dart_expand_root_noalloc(const dart_config* cfg, const void* E, c
 
     SelectArgs sa;
     std::memset(&sa, 0, sizeof sa);
-    sa.N = N;
     sa.P = 1;
     sa.k = c.k;
     sa.nV = nV;

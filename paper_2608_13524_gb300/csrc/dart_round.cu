@@ -425,7 +425,6 @@ __device__ void select_sequence(const RoundArgs& a, SelectArgs& sa, int dep, int
     const int prev_count = dep == 1 ? 1 : __ldcg(a.tree_count + s * a.L + dep - 2);
     merge_nodes(a, s, P, prev_count, stage);
     __syncthreads();
-    sa.N = N;
     sa.P = P;
     sa.dep = dep;
     sa.Pn = Pn;
@@ -972,7 +971,6 @@ __global__ void __launch_bounds__(kRoundThreads, 1) round_cluster_f32_kernel(con
         cluster_sync_all();
         // B2: the frontier (and after depth L prune and emit), rank 0
         if (rank == 0) {
-            sa.N = a.nseq * P;
             sa.P = P;
             sa.dep = dep;
             sa.Pn = Pn;
