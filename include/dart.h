@@ -243,8 +243,19 @@ int dart_build_chain_ddtree(dart_handle *h, const float *drafter_logits, const f
  * of its children q~_{d+1}(. | u_1..u_d) over the vocabulary (none at depth
  * L).  For beta <= 0 the result is the top-B of ALL prefixes by Eq. 5.
  * Emitted in pop order.  Needs DART_VARIANT_SEQ_HEAP in cfg.variants (else
- * DART_ERR_STATE).  Cost: up to B LM-head passes of one node per sequence,
- * one after another.  Cached as a CUDA graph like dart_build_tree. */
+ * DART_ERR_STATE).  An LM-head pass costs about the same for one prefix
+ * as for a node group, so each pass also corrects the prefixes that the
+ * search is likely to pop next: up to M = 16 / nseq per sequence (4 / nseq
+ * with fp32 weights, at least 1); the rows are those of the search that
+ * corrects one at a time.  Cost: as many passes, one after another, as the
+ * search needs (at most B - 1 and one for the root; about six for 64 nodes of
+ * depth 16).  Cached as a CUDA graph like dart_build_tree, whose passes are
+ * the body of a conditional node; when the caller captures the stream (and
+ * while profiling) all B passes are launched one after another, and those
+ * that find nothing to correct still run their kernels (with bf16 weights
+ * the LM-head streams E).  Workspace per sequence: 2 B + M states and child
+ * lists of min(B, V) tokens, values and links (B + 1 where M = 1), and M rows
+ * of V scaled logits. */
 int dart_build_seq_heap(dart_handle *h, const float *drafter_logits, const float *anchor_h,
                         const dart_tree_out *out, void *stream);
 
@@ -335,7 +346,7 @@ int dart_profile_read(dart_handle *h, float *lmhead_ms, int *lmhead_launches);
  * (cand_k > 0, once per round), 10 candidate scoring (cand_k > 0, per
  * depth), 11 gather of the per-token table row + SiLU + split (split first
  * layer), 12 top-K by value over a row of scaled logits (the best-first
- * constructions), 13 DDTree search, 14 one pop of the sequential search,
+ * constructions), 13 DDTree search, 14 one step of the sequential search,
  * 15 its emission, 16 the fused small-problem round (fused_round: one
  * launch per round), 17 the early L2 prefetch of the next depth's first E
  * tiles (side stream), 18 the starting bound of the top-k filters
