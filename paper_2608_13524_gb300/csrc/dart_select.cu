@@ -106,8 +106,10 @@ __device__ __forceinline__ void append_reaching(const uint64_t* keys, int n, uin
 }
 
 // npb nodes per block: block r of a cluster merges the nodes r * npb ...
+// (One block per SM at least: left to itself the compiler may keep two blocks of
+// threads by 32 registers a thread and spill, 3 x 11 nodes 493 -> 522 µs per round.)
 template <int kPer>
-__global__ void __launch_bounds__(kMergeThreads) merge_select_kernel(const SelectArgs a, int cs, int npb) {
+__global__ void __launch_bounds__(kMergeThreads, 1) merge_select_kernel(const SelectArgs a, int cs, int npb) {
     pdl_trigger();
     cluster_started_arrive();
     constexpr int kNodes = kMergeThreads / kPer, kWarps = kPer / 32;
