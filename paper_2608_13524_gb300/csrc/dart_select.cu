@@ -106,9 +106,17 @@ __device__ __forceinline__ void append_reaching(const uint64_t* keys, int n, uin
 }
 
 // npb nodes per block: block r of a cluster merges the nodes r * npb ...
+// kFew: fewer lists than k (small vocabularies, large k), where no list head
+// bounds the k-th key and a thread that walked its list would wait for a round
+// trip per four keys.  The threshold then is the r-th largest of the lists'
+// j-th keys, j the least with j * nV >= k and r = ceil(k / j): at least r * j
+// keys reach it; and the node's keys, at most 63 * 64, are read eight per
+// thread at once.  Measured on GB300 (µs, events around the launch; walking the
+// lists, now): 10 nodes, k = 61, 49 lists 37.8, 15.3; 6 x 3 nodes, k = 57, 20
+// lists 56.0, 11.0; 2 x 6 nodes, k = 41, 23 lists 41.5, 13.1.
 // (One block per SM at least: left to itself the compiler may keep two blocks of
 // threads by 32 registers a thread and spill, 3 x 11 nodes 493 -> 522 µs per round.)
-template <int kPer>
+template <int kPer, bool kFew>
 __global__ void __launch_bounds__(kMergeThreads, 1) merge_select_kernel(const SelectArgs a, int cs, int npb) {
     pdl_trigger();
     cluster_started_arrive();
@@ -145,8 +153,29 @@ __global__ void __launch_bounds__(kMergeThreads, 1) merge_select_kernel(const Se
         const uint64_t* lists = a.part_key + static_cast<size_t>(n) * stride;
         const float2 m0 = mine && tid < a.nV ? __ldcg(ms + tid) : none;
         const float2 m1 = mine && tid + kPer < a.nV ? __ldcg(ms + tid + kPer) : none;
-        uint64_t v[4] = {0ull, 0ull, 0ull, 0ull};
-        if (mine && tid < a.nV) load4(lists + tid * a.klist, a.klist, wide, v);
+        constexpr int kKeys = kFew ? 8 : 4;  // keys of this thread
+        uint64_t v[kKeys] = {};
+        uint64_t g = 0ull;  // the key whose rank gives the threshold
+        const int jth = kFew ? (a.k + a.nV - 1) / a.nV : 1;
+        // (kFew: the node's keys i0 + 2 * (tid + u * kPer) and the next, u < 4)
+        auto load_keys = [&](int i0) {
+#pragma unroll
+            for (int u = 0; u < kKeys / 2; u++) {
+                const int i = i0 + 2 * (tid + u * kPer);
+                ulonglong2 x = make_ulonglong2(0ull, 0ull);
+                if (mine && i < a.nV * a.klist) x = __ldcg(reinterpret_cast<const ulonglong2*>(lists + i));
+                v[2 * u] = x.x;
+                v[2 * u + 1] = i + 1 < a.nV * a.klist ? x.y : 0ull;  // (an odd number of keys: past the end)
+            }
+        };
+        if constexpr (kFew) {
+            if (mine && tid < a.nV)
+                g = __ldcg(reinterpret_cast<const unsigned long long*>(lists) + tid * a.klist + jth - 1);
+            load_keys(0);
+        } else {
+            if (mine && tid < a.nV) load4(lists + tid * a.klist, a.klist, wide, v);
+            g = v[0];
+        }
         const uint64_t bound =
             a.gthr && mine ? __ldcg(reinterpret_cast<const unsigned long long*>(a.gthr) + n) : 0ull;
         const float ps = a.dep == 1 || !mine
@@ -163,9 +192,8 @@ __global__ void __launch_bounds__(kMergeThreads, 1) merge_select_kernel(const Se
         // heads are dealt into 2^q >= k groups, each of whose maxima reaches
         // the least of them; above: the k-th largest head.  (Lists past kPer,
         // which only candidate sets of more than 512 tokens have, are left out.)
-        const bool groups = a.k <= kGroupMaxK;
+        const bool groups = !kFew && a.k <= kGroupMaxK;
         const int q2 = a.k <= 1 ? 1 : 1 << (32 - __clz(a.k - 1));
-        uint64_t g = v[0];
         if (groups) {
 #pragma unroll 1
             for (int o = 16; o >= q2; o >>= 1) {
@@ -194,7 +222,7 @@ __global__ void __launch_bounds__(kMergeThreads, 1) merge_select_kernel(const Se
             }
         } else {
             const int nl = min(a.nV, kPer);
-            if (v[0] != 0ull && count_above(heads, nl, v[0]) == a.k - 1) thr2[half] = v[0];
+            if (g != 0ull && count_above(heads, nl, g) == (a.k + jth - 1) / jth - 1) thr2[half] = g;
             __syncthreads();
             T = thr2[half];
         }
@@ -206,13 +234,22 @@ __global__ void __launch_bounds__(kMergeThreads, 1) merge_select_kernel(const Se
                 if (pos < kRankMax) surv[pos] = x;
                 return true;
             };
-            bool more = take(v[0]) && take(v[1]) && take(v[2]) && take(v[3]);
+            if constexpr (kFew) {
 #pragma unroll 1
-            for (int r = tid, j = 4; mine && r < a.nV; r += kPer, j = 0, more = true) {
+                for (int i0 = 0; i0 < a.nV * a.klist; i0 += kKeys * kPer) {
+                    if (i0 > 0) load_keys(i0);
+#pragma unroll
+                    for (int u = 0; u < kKeys; u++) take(v[u]);
+                }
+            } else {
+                bool more = take(v[0]) && take(v[1]) && take(v[2]) && take(v[3]);
 #pragma unroll 1
-                for (; more && j < a.klist; j += 4) {
-                    load4(lists + r * a.klist + j, a.klist - j, wide, v);
-                    more = take(v[0]) && take(v[1]) && take(v[2]) && take(v[3]);
+                for (int r = tid, j = 4; mine && r < a.nV; r += kPer, j = 0, more = true) {
+#pragma unroll 1
+                    for (; more && j < a.klist; j += 4) {
+                        load4(lists + r * a.klist + j, a.klist - j, wide, v);
+                        more = take(v[0]) && take(v[1]) && take(v[2]) && take(v[3]);
+                    }
                 }
             }
         }
@@ -579,8 +616,9 @@ int merge_select_smem(int P, int nV, int k) { return merge_plan(P, nV, k).smem; 
 
 cudaError_t select_set_smem_limits() {
     cudaError_t e = cudaSuccess;
-    for (const void* fn : {reinterpret_cast<const void*>(merge_select_kernel<256>),
-                           reinterpret_cast<const void*>(merge_select_kernel<512>)}) {
+    for (const void* fn : {reinterpret_cast<const void*>(merge_select_kernel<256, false>),
+                           reinterpret_cast<const void*>(merge_select_kernel<512, false>),
+                           reinterpret_cast<const void*>(merge_select_kernel<256, true>)}) {
         if (e == cudaSuccess) e = set_max_dynamic_smem(fn);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     }
@@ -589,7 +627,9 @@ cudaError_t select_set_smem_limits() {
 
 cudaError_t launch_merge_select(const SelectArgs& a, cudaStream_t st) {
     const MergePlan m = merge_plan(a.P, a.nV, a.k);
-    return launch_pdl_cluster(m.per == 256 ? merge_select_kernel<256> : merge_select_kernel<512>,
+    return launch_pdl_cluster(a.nV < a.k     ? merge_select_kernel<256, true>  // (k <= 64: m.per is 256)
+                              : m.per == 256 ? merge_select_kernel<256, false>
+                                             : merge_select_kernel<512, false>,
                               dim3(a.nseq * m.cs), dim3(m.nh * m.per), m.smem, st, m.cs, a, m.cs, m.npb);
 }
 

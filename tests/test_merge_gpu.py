@@ -84,3 +84,43 @@ def test_merge_select(dart, nseq, V, W, k, cand_k, pattern):
                 prev[s] = [-t[0] for t in top]
     finally:
         eng.close()
+
+
+# fewer vocabulary ranges than k: one, k - 1, an odd number of keys in all, more than are read at
+# once (63 lists of 64), ties, keys that are few or dense enough for the radix fallback, k <= 16
+FEW = [(1, 100, 8, 64, 0, "normal"), (2, 63 * 128, 8, 64, 0, "normal"), (1, 48 * 128, 64, 49, 0, "ties"),
+       (1, 33 * 128 - 5, 17, 63, 0, "normal"), (3, 20 * 128, 3, 57, 0, "normal"), (1, 40 * 128, 16, 61, 0, "dense"),
+       (1, 12 * 128, 4, 40, 0, "sparse"), (2, 5 * 128 + 1, 9, 9, 0, "ties")]
+
+
+@pytest.mark.parametrize("nseq,V,W,k,cand_k,pattern", FEW)
+def test_merge_select_fewer_lists_than_k(dart, nseq, V, W, k, cand_k, pattern):
+    test_merge_select(dart, nseq, V, W, k, cand_k, pattern)
+
+
+def test_few_lists_cost_no_more_than_many(dart):
+    """Fewer lists than k hold fewer keys than many do: merging them takes no
+    longer (a thread that walks its list waits for a round trip per four keys:
+    four times as long at 20 lists of 57)."""
+    us = {}
+    for V in (20 * 128, 150 * 128):
+        cfg = Config("few", 2, V, 64, 4, 3, 57, 8, "bf16", 0.0, 1)
+        g = np.random.Generator(np.random.PCG64(V))
+        t = lambda a, dt: torch.from_numpy(a.astype(np.float32)).to(dt).cuda()  # noqa: E731
+        eng = dart.Dart(cfg, t(g.standard_normal((64, 128)) * 0.1, torch.bfloat16),
+                        t(g.standard_normal((64, 64)) * 0.1, torch.bfloat16),
+                        t(g.standard_normal((V, 64)) * 0.02, torch.bfloat16))
+        D, h0 = t(g.standard_normal((2, 4, V)) * 3, torch.float32), t(g.standard_normal((2, 64)), torch.float32)
+        try:
+            dart.dart_set_profiling(eng.h, True)
+            eng.build_tree(D, h0)
+            dart.dart_profile_read_kinds(eng.h)
+            for _ in range(5):
+                eng.build_tree(D, h0)
+            ms, n = dart.dart_profile_read_kinds(eng.h)["merge_select"]
+            assert dart.dart_status_sync(eng.h) == 0
+        finally:
+            eng.close()
+        us[V] = ms / n * 1e3
+    print(us)
+    assert us[20 * 128] < 1.5 * us[150 * 128], us
