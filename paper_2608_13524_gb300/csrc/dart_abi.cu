@@ -69,6 +69,7 @@ int ng_index(int NG) { return NG == 16 ? 0 : (NG == 32 ? 1 : (NG == 64 ? 2 : 3))
 struct DepthPlan {
     int N, P, NG, G, nV, stages, smem;  // LM-head scoring
     int pair;                            // LM-head: CTA pairs
+    int cap;                             // LM-head: candidate slots per node
     int l2pf;                            // LM-head: E tiles per CTA prefetched into L2 before its wait
     int epf;                             // of those and the stages, how many the previous depth prefetches early
     int bound;                           // seed rows per sequence of the seed pass before this depth's LM-head (0: none)
@@ -385,8 +386,29 @@ int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, st
         p.P = caps[dep - 1];
         p.N = c.nseq * p.P;
         if (tc) {
+            // The LM-head offers a logit to a node's top-k merges only if it
+            // beats the node's filter bound; at k >= 32 the merges of the
+            // first tiles (where the bound is still low) limit the kernel,
+            // and a small kernel that bounds each node's k-th best score
+            // from the rows of largest drafter logit lets the filter start
+            // high (csrc/dart_bound.cu).
+            // Measured on GB300 (µs per round, same box, AUTO's choice in
+            // brackets): 64 nodes, k = 64: 3421 -> 2706 [on]; 64 nodes
+            // (4 x 16), k = 16: 2743 -> 2664 [on]; 256 nodes (8 x 32),
+            // k = 32: 9594 -> 8670 [on; 128 seed rows: 8964]; 256 nodes,
+            // k = 8: 8495 -> 8286 [on]; 32 nodes, k = 32: 2520 -> 2518
+            // [off]; 16 nodes, k = 16: 3415 -> 3475 [off].  The candidate
+            // slots per node depend on it (plan_lmhead_tc).
+            const int bR = std::max(64, (2 * c.k + 63) / 64 * 64);
+            const int bstat = seed_score_static_smem();
+            const bool want = c.topk_bound == DART_ON || (c.topk_bound == DART_AUTO && p.N > 32);
+            p.bound = (want && c.cand_k == 0 && bR <= kBoundR && c.V >= bR && bstat >= 0 &&
+                       seed_score_smem(c.d) + bstat <= static_cast<size_t>(h->smem_optin))
+                          ? bR
+                          : 0;
             LmheadPlan lp;
-            if (!plan_lmhead_tc(p.N, c.V, c.d, c.k, h->num_sms, h->smem_optin, c.lmhead_ctas_per_sm, h->tiled, &lp))
+            if (!plan_lmhead_tc(p.N, c.V, c.d, c.k, h->num_sms, h->smem_optin, c.lmhead_ctas_per_sm, h->tiled,
+                                p.bound > 0, &lp))
                 return DART_ERR_UNSUPPORTED;
             p.NG = lp.NG;
             p.G = lp.G;
@@ -394,6 +416,7 @@ int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, st
             p.stages = lp.stages;
             p.smem = lp.smem;
             p.pair = lp.pair ? 1 : 0;
+            p.cap = lp.cap;
             // One group of <= 16 nodes: every CTA streams its own slice of
             // E and the launch is HBM-bound.  Besides the stages it loads
             // before waiting on the previous kernel (which is latency-bound
@@ -418,27 +441,6 @@ int build_plans(dart_handle* h, const dart_config& c, std::vector<int>& caps, st
             p.epf = (p.l2pf > 0 && free_l2 > 0)
                         ? static_cast<int>(std::min<long long>(free_l2 / per_unit, p.stages + p.l2pf))
                         : 0;
-            // The LM-head offers a logit to a node's top-k merges only if it
-            // beats the node's filter bound; at k >= 32 the merges of the
-            // first tiles (where the bound is still low) limit the kernel,
-            // and a small kernel that bounds each node's k-th best score
-            // from the rows of largest drafter logit lets the filter start
-            // high (csrc/dart_bound.cu).
-            // Measured on GB300 (µs per round, same box, AUTO's choice in
-            // brackets): 64 nodes, k = 64: 3421 -> 2706 [on]; 64 nodes
-            // (4 x 16), k = 16: 2743 -> 2664 [on]; 256 nodes (8 x 32),
-            // k = 32: 9594 -> 8670 [on; 128 seed rows: 8964]; 256 nodes,
-            // k = 8: 8495 -> 8286 [on]; 32 nodes, k = 32: 2520 -> 2518
-            // [off]; 16 nodes, k = 16: 3415 -> 3475 [off].  64-node
-            // groups keep 32 candidate slots per node, 128-node groups 16,
-            // which needs the bound (without it: +6 % at 64 nodes, k = 64).
-            const int bR = std::max(64, (2 * c.k + 63) / 64 * 64);
-            const int bstat = seed_score_static_smem();
-            const bool want = c.topk_bound == DART_ON || (c.topk_bound == DART_AUTO && p.N > 32);
-            p.bound = (want && c.cand_k == 0 && bR <= kBoundR && c.V >= bR && bstat >= 0 &&
-                       seed_score_smem(c.d) + bstat <= static_cast<size_t>(h->smem_optin))
-                          ? bR
-                          : 0;
         } else {
             p.NG = pick_ng_f32(p.N);
             p.G = (p.N + p.NG - 1) / p.NG;
@@ -859,6 +861,7 @@ LmheadArgs lmhead_args(const dart_handle* h, const dart_config& c, const DepthPl
     la.bhalf = kNPadMax;
     la.stages = p.stages;
     la.pair = p.pair;
+    la.cap = p.cap;
     la.l2pf = p.l2pf;
     la.part_ms = h->part_ms;
     la.part_key = h->part_key;

@@ -116,6 +116,7 @@ struct LmheadArgs {
     uint64_t* gthr;       // [N] cross-CTA top-k bounds, zero before the launch (may be null)
     int e_tiled;          // the E tensor map is over the tiled copy (launch_retile), not [V][d]
     int pair;             // launch as CTA pairs (LmheadPlan)
+    int cap;              // candidate slots per node (LmheadPlan)
     int DS;               // fp32 kernel: blocks (one cluster) sharing a vocabulary range, each a slice of d
     // optional (null: unused)
     const int* dlog_row;  // [N / P] drafter row of each sequence's nodes (replaces dlog_row_off / V)
@@ -157,7 +158,7 @@ cudaError_t launch_gemm_tc(const CUtensorMap* tmA, const CUtensorMap* tmB, const
                            cudaStream_t st);
 int tc_stage_bytes(int NG);
 int lmhead_tc_tmem_cols(int NG);  // TMEM columns one LM-head CTA allocates
-int lmhead_tc_fixed_smem(int NG, int k, int stages);
+int lmhead_tc_fixed_smem(int NG, int k, int stages, int cap);
 int gemm_tc_fixed_smem(int stages);
 int lmhead_tc_ctas_per_sm(int NG, int smem);
 int gemm_tc_ctas_per_sm(int NG, int smem);
@@ -199,9 +200,10 @@ cudaError_t launch_lmhead_l2_prefetch(const CUtensorMap* tmE, int tiles, int nV,
 struct LmheadPlan {
     int NG, G, nV, stages, smem;
     bool pair;  // two neighbouring vocabulary ranges as a CTA pair
+    int cap;    // candidate slots per node
 };
 bool plan_lmhead_tc(int N, int V, int d, int k, int num_sms, int smem_optin, int ctas_per_sm_pref, bool e_tiled,
-                    LmheadPlan* out);
+                    bool bounded, LmheadPlan* out);  // bounded: the filters start from a bound (topk_bound)
 
 // fp32 CUDA-core kernels (dart_f32.cu)
 cudaError_t launch_lmhead_f32(const LmheadArgs& a, cudaStream_t st);

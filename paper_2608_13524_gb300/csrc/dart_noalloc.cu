@@ -143,7 +143,7 @@ extern "C" int dart_expand_root_noalloc(const dart_config* cfg, const void* E, c
     // and a row-major E (this entry point keeps no tiled copy)
     const int N = c.nseq;
     LmheadPlan lp;
-    if (!plan_lmhead_tc(N, c.V, c.d, c.k, ds.sms, ds.optin, c.lmhead_ctas_per_sm, false, &lp) || lp.G != 1)
+    if (!plan_lmhead_tc(N, c.V, c.d, c.k, ds.sms, ds.optin, c.lmhead_ctas_per_sm, false, false, &lp) || lp.G != 1)
         return DART_ERR_UNSUPPORTED;
     const int NG = lp.NG, nV = lp.nV;
     const int tiles = (c.V + kTileM - 1) / kTileM;
@@ -196,6 +196,7 @@ extern "C" int dart_expand_root_noalloc(const dart_config* cfg, const void* E, c
     la.bhalf = kBhalfNoAlloc;
     la.stages = lp.stages;
     la.pair = lp.pair ? 1 : 0;
+    la.cap = lp.cap;
     la.part_ms = part_ms;
     la.part_key = part_key;
     la.status = status;

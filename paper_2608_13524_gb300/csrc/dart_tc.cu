@@ -49,11 +49,19 @@ constexpr int epi_chunks() {
 // a tile rarely offers more than a few logits per node.  Measured on GB300
 // at 64 nodes, k = 64 (µs per round, same box): 128 slots 3042, 64 slots
 // 2806, 32 slots 2706 with the bound; without it 32 slots cost +6 %.  128-node
-// groups keep 16, which makes room for a fifth stage (389 instead of 403 µs
-// per launch at 256 nodes; 8 slots change nothing more).
+// groups keep 16 (cand_slots), which makes room for a fifth stage (389 instead
+// of 403 µs per launch at 256 nodes; 8 slots change nothing more), but 32 where
+// tiles offer more: without the bound, and in ranges of one tile.
+// Measured on GB300 (µs per round of 3 depths at d = 5120, where there is no
+// bound, and 4 at d = 4096; 16 slots, 32): 8 x 32 nodes, k = 32, V = 151936,
+// d = 5120 1628, 1579; 16 x 6, k = 34, V = 30000, d = 5120 561, 465; 8 x 32, k = 32,
+// d = 4096 V = 600 472, 451, V = 12000 485, 485, V = 32000 628, 646.
 template <int NG>
 constexpr int lm_cand_cap() {
-    return NG > 64 ? kCandCapLarge / 2 : NG == 64 ? kCandCapLarge : kCandCap;
+    return NG >= 64 ? kCandCapLarge : kCandCap;
+}
+int cand_slots(int NG, bool bounded, bool one_tile) {
+    return NG > 64 && bounded && !one_tile ? kCandCapLarge / 2 : NG >= 64 ? kCandCapLarge : kCandCap;
 }
 template <int NG>
 constexpr int threads() {
@@ -485,7 +493,8 @@ constexpr int lm_tmem_cols() {
 // of every sum are those of the single CTAs.  Measured on GB300, 256 nodes,
 // V = 151936, d = 4096 (µs per launch): single CTAs 450 (0.45 µs per k-block,
 // 107 GB/s into each SM), pairs with 4 stages 403, with 5 389.
-template <int NG, bool kPair>
+// (kCap: candidate slots per node, cand_slots)
+template <int NG, bool kPair, int kCap = lm_cand_cap<NG>()>
 __global__ void __launch_bounds__(threads<NG>(), 1)
     lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmE, const __grid_constant__ CUtensorMap tmH,
                      const LmheadArgs a) {
@@ -494,7 +503,6 @@ __global__ void __launch_bounds__(threads<NG>(), 1)
     const int stages = a.stages;
     constexpr int kNacc = lm_nacc<NG>();
     Smem s = carve<NG, kPair>(smem_raw, stages, kNacc);
-    constexpr int kCap = lm_cand_cap<NG>();
     EpiSmem e;
     e.cap = kCap;
     e.list = reinterpret_cast<uint64_t*>(s.tail);
@@ -825,8 +833,8 @@ __global__ void __launch_bounds__(threads<NG>(), 2)
 }
 
 template <int NG>
-int lmhead_fixed(int k, int stages) {
-    return (2 * stages + 2 * lm_nacc<NG>() + 1) * 8 + 16 + NG * k * 8 + NG * lm_cand_cap<NG>() * 8 + NG * 8 + 4 * NG * 8 + 4 * NG * 4 +
+int lmhead_fixed(int k, int stages, int cap) {
+    return (2 * stages + 2 * lm_nacc<NG>() + 1) * 8 + 16 + NG * k * 8 + NG * cap * 8 + NG * 8 + 4 * NG * 8 + 4 * NG * 4 +
            NG * 4 + 8;
 }
 
@@ -863,9 +871,13 @@ template <int NG>
 cudaError_t launch_lmhead_ng(const CUtensorMap* tmE, const CUtensorMap* tmH, const LmheadArgs& a, int smem,
                              cudaStream_t st) {
     if constexpr (NG == 128) {
+        constexpr int kFew = kCandCapLarge / 2;
         if (a.pair)
-            return launch_pdl_cluster(lmhead_tc_kernel<NG, true>, dim3(a.nV * a.G), dim3(threads<NG>()), smem, st, 2,
-                                      *tmE, *tmH, a);
+            return launch_pdl_cluster(a.cap == kFew ? lmhead_tc_kernel<NG, true, kFew> : lmhead_tc_kernel<NG, true>,
+                                      dim3(a.nV * a.G), dim3(threads<NG>()), smem, st, 2, *tmE, *tmH, a);
+        if (a.cap == kFew)
+            return launch_pdl(lmhead_tc_kernel<NG, false, kFew>, dim3(a.nV * a.G), dim3(threads<NG>()), smem, st, *tmE,
+                              *tmH, a);
     }
     return launch_pdl(lmhead_tc_kernel<NG, false>, dim3(a.nV * a.G), dim3(threads<NG>()), smem, st, *tmE, *tmH, a);
 }
@@ -912,12 +924,12 @@ int lmhead_tc_tmem_cols(int NG) {
     }
 }
 
-int lmhead_tc_fixed_smem(int NG, int k, int stages) {
+int lmhead_tc_fixed_smem(int NG, int k, int stages, int cap) {
     switch (NG) {
-        case 16: return lmhead_fixed<16>(k, stages) + 1024;
-        case 32: return lmhead_fixed<32>(k, stages) + 1024;
-        case 64: return lmhead_fixed<64>(k, stages) + 1024;
-        default: return lmhead_fixed<128>(k, stages) + 1024;
+        case 16: return lmhead_fixed<16>(k, stages, cap) + 1024;
+        case 32: return lmhead_fixed<32>(k, stages, cap) + 1024;
+        case 64: return lmhead_fixed<64>(k, stages, cap) + 1024;
+        default: return lmhead_fixed<128>(k, stages, cap) + 1024;
     }
 }
 
@@ -975,7 +987,7 @@ int lmhead_tc_ctas_per_sm(int NG, int smem) {
 constexpr int kLmheadPairNG = 128;
 
 bool plan_lmhead_tc(int N, int V, int d, int k, int num_sms, int smem_optin, int ctas_per_sm_pref, bool e_tiled,
-                    LmheadPlan* out) {
+                    bool bounded, LmheadPlan* out) {
     LmheadPlan p;
     p.NG = N <= 16 ? 16 : (N <= 32 ? 32 : (N <= 64 ? 64 : 128));
     p.G = (N + p.NG - 1) / p.NG;
@@ -985,7 +997,8 @@ bool plan_lmhead_tc(int N, int V, int d, int k, int num_sms, int smem_optin, int
     const int nv1 = std::max(1, std::min(num_sms / p.G, tiles));
     p.pair = p.NG >= kLmheadPairNG && nv1 % 2 == 0;
     const int sb = p.pair ? kATileBytes + p.NG * 128 : tc_stage_bytes(p.NG);
-    const int fixed = lmhead_tc_fixed_smem(p.NG, k, 16);
+    p.cap = cand_slots(p.NG, bounded, nv1 >= tiles);
+    const int fixed = lmhead_tc_fixed_smem(p.NG, k, 16, p.cap);
     auto stages_in = [&](int budget) { return std::min(16, (budget - fixed) / sb); };
     // Two CTAs per SM when both fit with >= 4 pipeline stages each: two
     // independent TMA streams per SM, and one CTA's epilogue / start-up /
@@ -995,7 +1008,7 @@ bool plan_lmhead_tc(int N, int V, int d, int k, int num_sms, int smem_optin, int
     // contiguous 16 KB tiles two CTAs win at d = 4096 too (-3.6 % against
     // one CTA on the same tiles, -1.0 % against row-major with one).
     const int st2 = stages_in(smem_optin / 2 - 2048);
-    const int smem2 = lmhead_tc_fixed_smem(p.NG, k, st2) + st2 * sb;
+    const int smem2 = lmhead_tc_fixed_smem(p.NG, k, st2, p.cap) + st2 * sb;
     const bool want2 = ctas_per_sm_pref ? ctas_per_sm_pref == 2 : (e_tiled || d <= 3072);
     if (!p.pair && want2 && st2 >= 4 && 2 * lmhead_tc_tmem_cols(p.NG) <= 512 && lmhead_tc_ctas_per_sm(p.NG, smem2) >= 2) {
         p.stages = st2;
@@ -1004,7 +1017,7 @@ bool plan_lmhead_tc(int N, int V, int d, int k, int num_sms, int smem_optin, int
         p.stages = stages_in(smem_optin);
     }
     if (p.stages < 2) return false;
-    p.smem = lmhead_tc_fixed_smem(p.NG, k, p.stages) + p.stages * sb;
+    p.smem = lmhead_tc_fixed_smem(p.NG, k, p.stages, p.cap) + p.stages * sb;
     *out = p;
     return true;
 }
@@ -1020,6 +1033,8 @@ cudaError_t tc_set_smem_limits(int max_dyn) {
     DART_SET((lmhead_tc_kernel<64, false>))
     DART_SET((lmhead_tc_kernel<128, false>))
     DART_SET((lmhead_tc_kernel<128, true>))
+    DART_SET((lmhead_tc_kernel<128, false, kCandCapLarge / 2>))
+    DART_SET((lmhead_tc_kernel<128, true, kCandCapLarge / 2>))
     DART_SET(gemm_tc_kernel<16>)
     DART_SET(gemm_tc_kernel<32>)
     DART_SET(gemm_tc_kernel<64>)

@@ -39,3 +39,48 @@ def test_lmhead_pairs(dart, nseq, V, d, W, k, tiled):
     finally:
         eng.close()
     compare_with_oracle(cfg, ref, gst, g, tol_of(cfg), x=x)
+
+
+# 32 candidate slots per node (no starting bound, ranges of one tile) and 16, pairs and single CTAs
+SLOTS = [(8, 128 * 90, 64, 32, 40, 2), (8, 128 * 90, 64, 32, 40, 1), (3, 128 * 75, 128, 40, 64, 2),
+         (5, 128 * 31 + 5, 128, 13, 13, 2), (16, 128 * 160, 64, 6, 34, 2), (16, 128 * 5 - 3, 64, 6, 34, 1)]
+
+
+@pytest.mark.parametrize("nseq,V,d,W,k,bound", SLOTS)
+def test_candidate_slots(dart, nseq, V, d, W, k, bound):
+    cfg = Config("slots", nseq, V, d, 3, W, k, 60, "bf16", 0.0, 82, topk_bound=bound)
+    x = make_inputs(cfg)
+    dx = to_device(cfg, x)
+    ref = oracle.build_tree(cfg, x["Wi"], x["Wo"], x["E"], x["Dlog"], x["h0"])
+    eng = dart.Dart(cfg, dx["Wi"], dx["Wo"], dx["E"])
+    try:
+        g = tree_to_numpy(eng.build_tree(dx["Dlog"], dx["h0"]))
+        assert dart.dart_status_sync(eng.h) == 0
+        gst = gpu_supertree(dart, eng.h, cfg)
+    finally:
+        eng.close()
+    compare_with_oracle(cfg, ref, gst, g, tol_of(cfg), x=x)
+
+
+def test_slots_without_a_bound(dart):
+    """96 nodes without the starting bound: at 16 slots the merge rounds of the
+    first tiles made a pass 2.0 times as long as one of 64 nodes (32 slots)."""
+    us = {}
+    for W in (4, 6):
+        cfg = Config("slots-time", 16, 6000, 1024, 3, W, 34, 8, "bf16", 0.0, 83, topk_bound=2)
+        x = make_inputs(cfg)
+        dx = to_device(cfg, x)
+        eng = dart.Dart(cfg, dx["Wi"], dx["Wo"], dx["E"])
+        try:
+            dart.dart_set_profiling(eng.h, True)
+            eng.build_tree(dx["Dlog"], dx["h0"])
+            dart.dart_profile_read_kinds(eng.h)
+            for _ in range(5):
+                eng.build_tree(dx["Dlog"], dx["h0"])
+            ms, n = dart.dart_profile_read_kinds(eng.h)["lmhead"]
+            assert dart.dart_status_sync(eng.h) == 0
+        finally:
+            eng.close()
+        us[W] = ms / n * 1e3
+    print(us)
+    assert us[6] < 1.7 * us[4], us
