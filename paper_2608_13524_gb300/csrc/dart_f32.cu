@@ -366,6 +366,12 @@ cudaError_t launch_head_small_f32(int Nc, int d, const int* prow, const int* tok
         const cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(head_small_f32_kernel));
         if (e != cudaSuccess) return e;
     }
+    // (as the LM-head, where its weights take longer than a launch.  5 x 2 nodes,
+    // d = 1024, K = 204: 337 µs per round launched early, 187 now; 1 x 8 nodes,
+    // d = 512, K = 105: 113, 92)
+    if (d > 256)
+        return launch_after(head_small_f32_kernel, dim3(Nc * S), dim3(kHeadThreads), smem, st, S, d, S, prow, tok, h, E,
+                            Wi, Wo, eps, hnext);
     return launch_pdl_cluster(head_small_f32_kernel, dim3(Nc * S), dim3(kHeadThreads), smem, st, S, d, S, prow, tok,
                               h, E, Wi, Wo, eps, hnext);
 }

@@ -22,7 +22,8 @@ def dart():
 
 # candidate sets and large head GEMMs; the full vocabulary and many small head updates
 CASES = [Config("f32-cand", 4, 4000, 2048, 4, 39, 18, 60, "f32", 0.0, 95, cand_k=20),
-         Config("f32-full", 16, 30000, 768, 4, 5, 4, 20, "f32", 0.0, 96)]
+         Config("f32-full", 16, 30000, 768, 4, 5, 4, 20, "f32", 0.0, 96),
+         Config("f32-small-head", 5, 20502, 1024, 4, 2, 2, 8, "f32", 0.0, 97, cand_k=204)]
 
 
 @pytest.mark.parametrize("cfg", CASES, ids=lambda c: c.name)
