@@ -191,10 +191,17 @@ __device__ __forceinline__ void attn_drain(uint64_t* bar, uint32_t parity) {
     }
 }
 
+// Polls between two looks at the timer in tree_attn_kernel, whose eight softmax
+// warps wait together for every key tile and are better kept apart: with 32,
+// 0.5 to 1.2 % slower over long contexts (152 heads of 3 tiles, 8192 keys 217.0
+// and 219.4 µs), at no length faster.
+constexpr uint32_t kTilePolls = 1;
+
 // A wait whose outcome is the same for every lane of the warp (the
 // tcgen05.ld / st that follow are warp-collective).
+template <uint32_t kPolls = kWaitPolls>
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-    const bool got = mbar_wait_inline(bar, parity, abort);
+    const bool got = mbar_wait_inline<kPolls>(bar, parity, abort);
     return __all_sync(0xFFFFFFFFu, got);
 }
 
@@ -406,7 +413,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                 const int key0 = (ctx ? j : j - a.nct) * kKeys;
                 if (do_k) {
                     const int st = i % kKStages;
-                    if (!mbar_wait_inline(&k_empty[st], (static_cast<uint32_t>(i / kKStages) & 1u) ^ 1u, abort)) {
+                    if (!mbar_wait_inline<kTilePolls>(&k_empty[st], (static_cast<uint32_t>(i / kKStages) & 1u) ^ 1u, abort)) {
                         attn_timeout(a.status, abort);
                         break;
                     }
@@ -417,7 +424,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     kdone++;
                 } else {
                     const int st = i % kVStages;
-                    if (!mbar_wait_inline(&v_empty[st], (static_cast<uint32_t>(i / kVStages) & 1u) ^ 1u, abort)) {
+                    if (!mbar_wait_inline<kTilePolls>(&v_empty[st], (static_cast<uint32_t>(i / kVStages) & 1u) ^ 1u, abort)) {
                         attn_timeout(a.status, abort);
                         break;
                     }
@@ -446,12 +453,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (lane == 0 && nt > 0) {
             constexpr uint32_t idesc_s = idesc_bf16_f32(kRows, kKeys);
             constexpr uint32_t idesc_pv = idesc_bf16_f32(kRows, kDh) | (1u << 16);  // B (= V) MN-major
-            bool mok = mbar_wait_inline(q_ready, 0, abort);
+            bool mok = mbar_wait_inline<kTilePolls>(q_ready, 0, abort);
             auto issue_s = [&](int i) -> bool {
                 const int st = i % kKStages;
                 // the S columns were last read by softmax(i - 1)
-                if (!mbar_wait_inline(&k_full[st], static_cast<uint32_t>(i / kKStages) & 1u, abort) ||
-                    (i > 0 && !mbar_wait_inline(s_empty, static_cast<uint32_t>(i - 1) & 1u, abort)))
+                if (!mbar_wait_inline<kTilePolls>(&k_full[st], static_cast<uint32_t>(i / kKStages) & 1u, abort) ||
+                    (i > 0 && !mbar_wait_inline<kTilePolls>(s_empty, static_cast<uint32_t>(i - 1) & 1u, abort)))
                     return false;
                 tc_fence_after();
                 const uint32_t k_addr = smem_u32(sK + st * kTileBytes);
@@ -473,8 +480,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     break;
                 }
                 const int st = i % kVStages;
-                if (!mbar_wait_inline(p_full, static_cast<uint32_t>(i) & 1u, abort) ||
-                    !mbar_wait_inline(&v_full[st], static_cast<uint32_t>(i / kVStages) & 1u, abort)) {
+                if (!mbar_wait_inline<kTilePolls>(p_full, static_cast<uint32_t>(i) & 1u, abort) ||
+                    !mbar_wait_inline<kTilePolls>(&v_full[st], static_cast<uint32_t>(i / kVStages) & 1u, abort)) {
                     mok = false;
                     break;
                 }
@@ -507,7 +514,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             const float4* cs = reinterpret_cast<const float4*>(a.cs + (static_cast<size_t>(s) * a.B + min(b, a.B - 1)) * (kDh / 2));
 #pragma unroll
             for (int e = 0; e < 16; e++) f[e] = __ldg(cs + wg * 16 + e);
-            if (!warp_wait(q_full, 0, abort)) {
+            if (!warp_wait<kTilePolls>(q_full, 0, abort)) {
                 attn_timeout(a.status, abort);
                 ok = false;
             }
@@ -569,7 +576,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             // Both warps of the lane quarter reach both pair barriers of every
             // iteration and leave the loop at the same point: a failed wait is
             // exchanged with the row max and acted on after the barriers.
-            if (ok && !warp_wait(s_full, static_cast<uint32_t>(i) & 1u, abort)) {
+            if (ok && !warp_wait<kTilePolls>(s_full, static_cast<uint32_t>(i) & 1u, abort)) {
                 attn_timeout(a.status, abort);
                 ok = false;
             }
@@ -606,7 +613,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             // P buffer i & 1 was last read by PV(i - 2); O must be stable (PV(i - 1)
             // done) only when it is rescaled.  On a timeout this tile is
             // skipped; the pair leaves the loop together at the next exchange.
-            if (i > 1 && !warp_wait(&pv_done[i & 1], (static_cast<uint32_t>(i >> 1) & 1u) ^ 1u, abort)) {
+            if (i > 1 && !warp_wait<kTilePolls>(&pv_done[i & 1], (static_cast<uint32_t>(i >> 1) & 1u) ^ 1u, abort)) {
                 attn_timeout(a.status, abort);
                 ok = false;
                 continue;
@@ -614,7 +621,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             tc_fence_after();
             const bool any_resc = __any_sync(0xFFFFFFFFu, resc);
             if (i > 0 && any_resc) {
-                if (!warp_wait(&pv_done[(i - 1) & 1], static_cast<uint32_t>((i - 1) >> 1) & 1u, abort)) {
+                if (!warp_wait<kTilePolls>(&pv_done[(i - 1) & 1], static_cast<uint32_t>((i - 1) >> 1) & 1u, abort)) {
                     attn_timeout(a.status, abort);
                     ok = false;
                     continue;
@@ -655,7 +662,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             mbar_arrive(p_full);
         }
         if (ok && nt > 0) {
-            if (!warp_wait(&pv_done[(nt - 1) & 1], static_cast<uint32_t>((nt - 1) >> 1) & 1u, abort)) {
+            if (!warp_wait<kTilePolls>(&pv_done[(nt - 1) & 1], static_cast<uint32_t>((nt - 1) >> 1) & 1u, abort)) {
                 attn_timeout(a.status, abort);
                 ok = false;
             }
