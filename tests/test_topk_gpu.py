@@ -1,4 +1,4 @@
-"""Row top-K over several slices (a cluster of blocks per row) against the oracle:
+"""Row top-K over several slices (a block each, merged by the row's last block) against the oracle:
 rows that are not 16-byte aligned, more keys at the bound than are ranked at
 once (equal values, large K), rows of almost one value (radix select), infinities,
 and the by-value lists of the best-first constructions."""
